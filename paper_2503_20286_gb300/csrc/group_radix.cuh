@@ -41,7 +41,7 @@ __device__ bool radix_pass(const ProbDev& d, const Group& g, int gs, long long b
     __syncthreads();
     if (active)
         for (int i = tid; i < kRadix; i += blockDim.x) d.hist[g.rank * kRadix + i] = s_hist[i];
-    if (!group_sync(d.sc, g.size, budget)) return false;
+    if (!group_sync(g, d.sc, budget)) return false;
 
     // digit offsets of this CTA: all earlier digits + same digit of earlier CTAs
     if (tid == 0) s_skip = 0;
@@ -93,7 +93,7 @@ __device__ bool radix_pass(const ProbDev& d, const Group& g, int gs, long long b
             __syncthreads();
         }
     }
-    return group_sync(d.sc, g.size, budget);
+    return group_sync(g, d.sc, budget);
 }
 
 }  // namespace emo

@@ -148,7 +148,7 @@ __device__ __forceinline__ void hype_contributions(const Plan* plan, const Group
         __syncthreads();
         for (int64_t c = 1 + tid; c <= cmax; c += blockDim.x) alpha[c] = __ddiv_rn(alpha[c], (double)c);
     }
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // (D) contributions of the points of front l: one warp per point; the
     // samples and their weights alpha_{c_i} (0 beyond c = k, or when no point
@@ -203,7 +203,7 @@ __device__ __forceinline__ void hype_contributions(const Plan* plan, const Group
     if (in.hv_out)
         for (int64_t i = t0; i < n2; i += stride)
             if (__ldcg(&d.rank_o[i]) != l) in.hv_out[i] = 0.0;
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // (E) L by contribution descending (stable: ties keep the index order)
     if (want >= nL) {

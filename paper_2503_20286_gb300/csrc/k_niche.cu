@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_csr(Plan* plan)
         }
         d.loff[q] = lo;
     }
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
     for (int64_t t = t0; t < nL; t += stride) {
         const int j = __ldcg(&d.pi[__ldcg(&L[t])]);
         const int x = (int)(t - __ldcg(&d.loff[j])) + 1;
@@ -139,7 +139,7 @@ __device__ bool group_kth_key(const ProbDev& d, const Group& g, long long budget
     int32_t* hist = d.nhist;
     const int tid = threadIdx.x;
     for_keys([&](unsigned long long key) { atomicAdd(&hist[key >> 52], 1); });
-    if (!group_sync(sc, g.size, budget)) return false;
+    if (!group_sync(g, sc, budget)) return false;
 
     {  // the bin of the key of rank k (each thread scans 8 bins)
         constexpr int PER = kNicheBins / kCoopThreads;
@@ -168,7 +168,7 @@ __device__ bool group_kth_key(const ProbDev& d, const Group& g, long long budget
     for_keys([&](unsigned long long key) {
         if ((int)(key >> 52) == bin) d.ekeys[atomicAdd(&sc->ncol, 1)] = key;
     });
-    if (!group_sync(sc, g.size, budget)) return false;
+    if (!group_sync(g, sc, budget)) return false;
 
     const int nc = ld_volatile(&sc->ncol);  // the rank-kbin key among the collected ones
     if (nc <= kNicheSmallSel) {
@@ -419,7 +419,7 @@ __device__ bool niche_bulk(const ProbDev& d, const Group& g, long long budget, i
     const int bend = -block_reduce_min<kCoopThreads>(-cend, sm.warp);
     if (tid == 0) part[g.rank] = ((unsigned long long)(unsigned)bmin << 32) | (unsigned)bend;
     for (int64_t b = t0; b < kNicheBins; b += stride) hist[b] = 0;
-    if (!group_sync(sc, g.size, budget)) return false;
+    if (!group_sync(g, sc, budget)) return false;
     int lm = INT32_MAX, le = 0;
     for (int r = tid; r < g.size; r += blockDim.x) {
         const unsigned long long v = __ldcg(&part[r]);
@@ -444,7 +444,7 @@ __device__ bool niche_bulk(const ProbDev& d, const Group& g, long long budget, i
             if (r + n < R) atomicAdd(&hist[r + n], -1);
         }
     }
-    if (!group_sync(sc, g.size, budget)) return false;
+    if (!group_sync(g, sc, budget)) return false;
 
     // (3) every CTA: ne(c), P(c), c*, and the levels served up to c*
     {
@@ -507,10 +507,10 @@ __device__ bool niche_bulk(const ProbDev& d, const Group& g, long long budget, i
     const bool all = ne_star <= rem;
     unsigned long long thresh = ~0ull;
     if (!all) {  // the rem references of smallest priority among those at level c*
-        if (!group_sync(sc, g.size, budget)) return false;  // every CTA is done with the histogram
+        if (!group_sync(g, sc, budget)) return false;  // every CTA is done with the histogram
         for (int64_t b = t0; b < kNicheBins; b += stride) hist[b] = 0;
         if (g.rank == 0 && tid == 0) sc->ncol = 0;
-        if (!group_sync(sc, g.size, budget)) return false;
+        if (!group_sync(g, sc, budget)) return false;
         auto level_keys = [&](auto&& f) {
             for (int64_t j = t0; j < nr; j += stride) {
                 const int n = __ldcg(&d.lcnt[j]), r = __ldcg(&d.rho[j]);
@@ -560,7 +560,7 @@ __device__ bool niche_bulk(const ProbDev& d, const Group& g, long long budget, i
         d.lcnt[j] = n - take;
         d.rho[j] = r + take;
     }
-    if (!group_sync(sc, g.size, budget)) return false;
+    if (!group_sync(g, sc, budget)) return false;
     levels += s_lev;
     handled = found;
     remaining = found ? 0 : remaining - s_pwin;
@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_niche(Plan* plan)
         if (tid == 0) part[g.rank] = ((unsigned long long)(unsigned)bmin << 32) | (unsigned)bcnt;
         for (int64_t b = t0; b < kNicheBins; b += stride) hist[b] = 0;
         if (g.rank == 0 && tid == 0) sc->ncol = 0;
-        if (!group_sync(sc, g.size, budget)) return;
+        if (!group_sync(g, sc, budget)) return;
 
         // (B) the level: minimum c over the group and the number of references holding it
         int lm = INT32_MAX;
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_niche(Plan* plan)
             d.lcnt[j] = len - 1;
             d.rho[j] = c + 1;
         }
-        if (!group_sync(sc, g.size, budget)) return;
+        if (!group_sync(g, sc, budget)) return;
         remaining -= all ? ne : remaining;
         ++levels;
         if (remaining > 0 && levels >= kNicheDirectLevels) {  // the rest in bulk when the span allows
@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_niche_oneshot(Plan* plan)
         sc->ncol = 0;
         sc->levels = 1;
     }
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // (B) Update-Rank: add or drop in Philox order
     const int n_dif = K - ld_volatile(&sc->nsel);

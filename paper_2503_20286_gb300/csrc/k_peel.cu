@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
             atomicAdd(&d.sc->ranked, s_newn);
         }
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
 
     int64_t prev_total = 0, total = ld_volatile(&d.sc->ranked);
     int k = 0;
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
                 }
             }
         }
-        if (!group_sync(d.sc, g.size, budget)) return;
+        if (!group_sync(g, d.sc, budget)) return;
         prev_total = total;
         total = ld_volatile(&d.sc->ranked);
         ++k;
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel_wave(Plan* plan)
             s_k[i] = exhausted ? kInf : 0;
         }
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
 
     long long idle_since = clock64();
     for (;;) {
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel_wave(Plan* plan)
         }
         __syncthreads();
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
 
     // ---- results: l, |P|, |L| (set by the leader); ranks in caller order
     // (beyond l: not ranked); the list of S

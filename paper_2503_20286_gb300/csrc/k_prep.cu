@@ -257,12 +257,12 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
                 cur[j] = v;
             }
         }
-        if (!group_sync(d.sc, g.size, budget)) return;
+        if (!group_sync(g, d.sc, budget)) return;
         if (ld_volatile(&d.sc->longrun)) {  // full stable LSD sort from the index order
             int32_t* id = d.idx + (int64_t)(buf ^ 1) * d.n2p;
             for (int64_t s = (int64_t)g.rank * blockDim.x + threadIdx.x; s < n2; s += stride) id[s] = (int32_t)s;
             buf ^= 1;
-            if (!group_sync(d.sc, g.size, budget)) return;
+            if (!group_sync(g, d.sc, budget)) return;
             for (int k = m - 1; k >= 0; --k)
                 if (!sort_by(k)) return;
         }
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
         for (int w = 0; w < kCoopThreads / 32; ++w) mx = max(mx, s_warp[w]);
         d.hist[g.rank] = mx;
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
     __shared__ int s_carry;
     if (threadIdx.x == 0) {
         int c = 0;
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
     // every CTA has read the run-start carries from d.hist before the radix
     // passes of the references reuse it
     if (in.mode != MODE_SELECT) return;
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
     sort_references(d, g, budget, rsm);
 }
 

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
     }
     __syncthreads();
     if (tid < m && s_u32[tid]) atomicMax(&sc->zkey[tid], s_u32[tid]);
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
     if (tid < m) s_z[tid] = key_float(~__ldcg(&sc->zkey[tid]));
     if (tid < kMaxM) { s_u32[tid] = 0u; s_u64[tid] = 0ull; }
     __syncthreads();
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
         atomicMax(&sc->asf32[tid], s_u32[tid]);
         atomicMax(&sc->nadir[tid], s_u64[tid]);
     }
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // 3. exact FP64 ASF of the candidates within the FP32 error band
     if (tid < kMaxM) s_u64[tid] = 0ull;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
     }
     __syncthreads();
     if (tid < m) atomicMax(&sc->asf64[tid], s_u64[tid]);
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // 4. lowest index attaining the FP64 minimum (stored as INT32_MAX - i maxima)
     __shared__ unsigned long long s_best[kMaxM];
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
             if (asf32(v, j) <= s_lim[j] && dbits(asf64(v, j)) == s_best[j])
                 atomicMax(&sc->ext[j], INT32_MAX - (int)v);
     }
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
 
     // 5. intercepts by Gaussian elimination with partial pivoting (FP64)
     if (g.rank == 0 && tid == 0) {
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
     // 6. S in the order of the polar angle of its normalised points (16-bit
     // buckets, two radix passes): neighbouring threads of the association
     // then scan neighbouring references. Any order of S gives the same result.
-    if (!group_sync(sc, g.size, budget)) return;
+    if (!group_sync(g, sc, budget)) return;
     __shared__ RadixSmem rsm;
     float zf[kMaxM], ia[kMaxM];
     for (int k = 0; k < m; ++k) {
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
     }
     if (cur == 1) {
         for (int64_t i = t0; i < nS; i += stride) d.slist[i] = __ldcg(&d.llist[i]);
-        group_sync(sc, g.size, budget);
+        group_sync(g, sc, budget);
     }
 }
 

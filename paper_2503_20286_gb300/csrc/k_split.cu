@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_rank_in(Plan* plan)
         if (r < 0 || r >= n2) set_status(d.sc, EMO_ERR_INVALID_ARG);
         else atomicAdd(&d.wcnt[r], 1);
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
     if (g.rank == 0) {
         if (tid == 0) s_l = -1;
         int run = 0;
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_rank_in(Plan* plan)
             }
         }
     }
-    if (!group_sync(d.sc, g.size, budget)) return;
+    if (!group_sync(g, d.sc, budget)) return;
     const int l = ld_volatile(&d.sc->l);
     for (int64_t s0 = (int64_t)g.rank * blockDim.x; s0 < n2; s0 += stride) {
         const int64_t i = s0 + tid;
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_assoc_out(Plan* plan)
         sp.d_out[i - sp.col_lo] = inS ? __ldcg(&d.d64[i]) : (double)NAN;
         if (r < l) atomicAdd(&d.rho[p], 1);
     }
-    if (!group_sync(sc, g.size, plan->spin_budget)) return;
+    if (!group_sync(g, sc, plan->spin_budget)) return;
     for (int64_t j = t0; j < d.in.n_r; j += stride) sp.rho[j] = __ldcg(&d.rho[j]);
 }
 
