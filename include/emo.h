@@ -408,9 +408,11 @@ emo_status emo_standin_objectives(const float* X, int64_t n, int64_t d, int32_t 
 /*
  * Inverted generational distance: the mean over the n_ref points of `Ref`
  * of the distance to the nearest of the n points of F (squared distances in
- * float, square roots and the sum in double, summed in index order). F, Ref
- * device float [.][m]; igd_out device double; ws of
- * emo_workspace_size(EMO_OP_IGD, n_ref, m, 0) bytes (8-byte aligned).
+ * float, square roots and the sum in double, in a fixed order that depends on
+ * n_ref only). F, Ref device float [.][m]; igd_out device double; ws of
+ * emo_workspace_size(EMO_OP_IGD, n_ref, m, 0) bytes (8-byte aligned). With less
+ * workspace, down to 8 bytes per reference point, every pair is compared
+ * (the same result, more time).
  */
 emo_status emo_igd(const float* F, int64_t n, int32_t m, const float* Ref, int64_t n_ref, double* igd_out, void* ws,
                    size_t ws_bytes, emo_stream_t stream);

@@ -475,7 +475,7 @@ size_t emo_workspace_size(int op, int64_t n2, int32_t m, int32_t n_r)
         return b < 0 ? 0 : (size_t)(kPlanBytes + b);
     }
     if (op == EMO_OP_MOEAD_SELECT) return n_r >= 1 && n_r <= n2 ? (size_t)moead_layout(n2, m, n_r, nullptr, nullptr) : 0;
-    if (op == EMO_OP_IGD) return (size_t)(n2 * 8);
+    if (op == EMO_OP_IGD) return (size_t)igd_workspace(n2);
     int mode = op == EMO_OP_ND_RANK ? MODE_RANK
                : op == EMO_OP_NSGA3_SELECT ? MODE_SELECT
                : op == EMO_OP_HYPE_SELECT ? MODE_HYPE
@@ -637,7 +637,7 @@ emo_status emo_igd(const float* F, int64_t n, int32_t m, const float* Ref, int64
     if ((int64_t)ws_bytes < n_ref * 8) return EMO_ERR_WORKSPACE;
     DevInfo di = dev_info();
     if (!di.ok) return EMO_ERR_CUDA;
-    return launch_igd(F, n, m, Ref, n_ref, (double*)ws, igd_out, di.sms, (cudaStream_t)stream) == cudaSuccess
+    return launch_igd(F, n, m, Ref, n_ref, ws, (int64_t)ws_bytes, igd_out, di.sms, (cudaStream_t)stream) == cudaSuccess
                ? EMO_OK
                : EMO_ERR_CUDA;
 }

@@ -60,7 +60,10 @@ cudaError_t launch_variation(const VariationArgs& a, int sms, cudaStream_t s);
 cudaError_t launch_standin(const float* X, int64_t n, int64_t d, int m, int shape, float* F, int sms, cudaStream_t s);
 cudaError_t launch_gather_rows(const float* src, const int32_t* idx, int64_t rows, int64_t width, float* dst, int sms,
                                cudaStream_t s);
-cudaError_t launch_igd(const float* F, int64_t n, int m, const float* Ref, int64_t n_ref, double* dist, double* out,
-                       int sms, cudaStream_t s);
+// Workspace bytes of one IGD; with less (at least 8 per reference point) every
+// pair is compared.
+int64_t igd_workspace(int64_t n_ref);
+cudaError_t launch_igd(const float* F, int64_t n, int m, const float* Ref, int64_t n_ref, void* ws, int64_t ws_bytes,
+                       double* out, int sms, cudaStream_t s);
 
 }  // namespace emo
