@@ -22,7 +22,14 @@ using namespace emo;
 namespace {
 
 std::atomic<long long> g_spin_budget{0};
+constexpr int64_t cdiv_c(int64_t a, int64_t b) { return (a + b - 1) / b; }
 constexpr int kPeelDynSmem = peel_smem_bytes((int)(kMaxN2 / kColBlock));
+// k_fronts: more than any size needs (the leaves' state is shared only up to
+// kFrontLeafSmem, where the nodes' is at most a 32nd of it)
+constexpr int kFrontsDynSmem = std::max((int)(cdiv_c(cdiv_c(kMaxN2, 32), 32) * kTreeMaxM * 4),
+                                        kFrontLeafSmem + kFrontLeafSmem / 32 + kTreeMaxM * 128) +
+                               std::max(front_local(3) * (4 + 32 * 4) * 4,
+                                        front_local(kTreeMaxM) * (4 + 32 * (kTreeMaxM + 1)) * 4);
 constexpr int kPeelWaveDynSmem = peel_wave_smem_bytes((int)(kMaxN2 / kColBlock));
 std::atomic<int> g_timing{0};
 
@@ -101,6 +108,8 @@ DevInfo dev_info()
                 cudaSuccess ||
             cudaFuncSetAttribute((const void*)k_peel_wave, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kPeelWaveDynSmem) != cudaSuccess ||
+            cudaFuncSetAttribute((const void*)k_fronts, cudaFuncAttributeMaxDynamicSharedMemorySize, kFrontsDynSmem) !=
+                cudaSuccess ||
             cudaFuncSetAttribute((const void*)k_hype_counts, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  hype_counts_smem(4)) != cudaSuccess)
             return DevInfo{};
@@ -109,11 +118,13 @@ DevInfo dev_info()
         const void* kernels[] = {(const void*)k_sort,  (const void*)k_peel,  (const void*)k_peel_wave,
                                  (const void*)k_stats, (const void*)k_csr,   (const void*)k_niche,
                                  (const void*)k_niche_oneshot, (const void*)k_hype, (const void*)k_finish,
-                                 (const void*)k_rank_in, (const void*)k_assoc_out, (const void*)k_given_in};
-        const int dyn[] = {0, kPeelDynSmem, kPeelWaveDynSmem, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+                                 (const void*)k_rank_in, (const void*)k_assoc_out, (const void*)k_given_in, (const void*)k_zorder,
+                                 (const void*)k_fronts};
+        const int dyn[] = {0, kPeelDynSmem, kPeelWaveDynSmem, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, kFrontsDynSmem};
         for (int i = 0; i < (int)(sizeof(dyn) / sizeof(dyn[0])); ++i) {
             int o = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernels[i], kCoopThreads, dyn[i]) != cudaSuccess)
+            const int threads = kernels[i] == (const void*)k_fronts ? kTreeThreads : kCoopThreads;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernels[i], threads, dyn[i]) != cudaSuccess)
                 return DevInfo{};
             occ = std::min(occ, o);
         }
@@ -150,10 +161,10 @@ ProbIn make_in(const float* F, const float* R, int64_t n2, int32_t m, int32_t n_
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
-cudaError_t coop(const void* fn, int G, size_t smem, cudaStream_t s, Plan* plan)
+cudaError_t coop(const void* fn, int G, size_t smem, cudaStream_t s, Plan* plan, int threads = kCoopThreads)
 {
     void* args[] = {&plan};
-    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kCoopThreads), args, smem, s);
+    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(threads), args, smem, s);
 }
 cudaError_t coop_phase(const void* fn, int G, size_t smem, cudaStream_t s, Plan* plan, int phase)
 {
@@ -315,7 +326,8 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     if (!ws || !aligned(ws, 256)) return EMO_ERR_INVALID_ARG;
     int64_t off = kPlanBytes;
     int max_ncb = 1;
-    bool any_select = false, any_hype = false;
+    int fronts_smem = 0;
+    bool any_select = false, any_hype = false, any_tree = false, any_matrix = false, any_lex = false;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return EMO_ERR_CUDA;
     for (auto& in : ins) {
@@ -328,6 +340,13 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         max_ncb = std::max<int>(max_ncb, (int)cdiv(in.n2, kColBlock));
         any_select |= in.mode == MODE_SELECT;
         any_hype |= in.mode == MODE_HYPE;
+        any_lex |= lex_ordered(in);
+        if (tree_ranked(in)) {
+            any_tree = true;
+            fronts_smem = std::max(fronts_smem, fronts_smem_bytes(in.n2, in.m));
+        } else {
+            any_matrix = true;
+        }
     }
     if ((int64_t)ws_bytes < off) return EMO_ERR_WORKSPACE;
 
@@ -348,7 +367,9 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     sm.mark("prep");
     // (from given ranks only the references are ordered; the niching from a
     // given association has none)
-    if (sp.kind != SPLIT_NICHE && coop((const void*)k_sort, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (sp.kind != SPLIT_NICHE && (any_lex || any_select) && coop((const void*)k_sort, di.G, 0, s, plan) != cudaSuccess)
+        return EMO_ERR_CUDA;
+    if (any_tree && coop((const void*)k_zorder, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("sort");
     if (nprob == 1 && ins[0].mode == MODE_DOM) {  // caller-order dominance matrix only
         const ProbIn& in = ins[0];
@@ -366,7 +387,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         sm.mark("rank_in");
         return run_selection_stages(ins, di, plan, dev, s, sm, true, sp.kind);
     }
-    if (launch_colprep(plan, di.sms, s, nprob) != cudaSuccess) return EMO_ERR_CUDA;
+    if (any_lex && launch_colprep(plan, di.sms, s, nprob) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("colprep");
     // dominance: one launch per objective count present
     long long item = 0;
@@ -374,17 +395,17 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         int q = p;
         long long hi = item;
         while (q < nprob && ins[q].m == ins[p].m) {
-            hi += dom_items_of(ins[q].n2, ins[q].dom_chunk);
+            if (!tree_ranked(ins[q])) hi += dom_items_of(ins[q].n2, ins[q].dom_chunk);
             ++q;
         }
-        if (launch_dominance_tri_range(ins[p].m, plan, di.sms, s, item, hi, &plan->dom_ctr[ins[p].m], p, q) !=
+        if (hi > item && launch_dominance_tri_range(ins[p].m, plan, di.sms, s, item, hi, &plan->dom_ctr[ins[p].m], p, q) !=
             cudaSuccess)
             return EMO_ERR_CUDA;
         item = hi;
         p = q;
     }
     sm.mark("dominance");
-    {
+    if (any_matrix) {
         int big = 0;
         for (int p = 1; p < nprob; ++p)
             if (ins[p].n2 > ins[big].n2) big = p;
@@ -393,6 +414,8 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         if (coop(wave ? (const void*)k_peel_wave : (const void*)k_peel, di.G, smem, s, plan) != cudaSuccess)
             return EMO_ERR_CUDA;
     }
+    if (any_tree && coop((const void*)k_fronts, di.G, (size_t)fronts_smem, s, plan, kTreeThreads) != cudaSuccess)
+        return EMO_ERR_CUDA;
     sm.mark("peel");
     if (any_select) {
         const emo_status st = run_selection_stages(ins, di, plan, dev, s, sm, false);
@@ -1040,7 +1063,7 @@ int32_t emo_device_report(char* buf, int32_t len)
     out += "; sms " + std::to_string(sms) + "; cooperative " + std::to_string(coop);
     DevInfo di = dev_info();  // also sets the dynamic shared memory limit of k_peel
     struct K { const char* name; const void* fn; int dyn; };
-    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_peel", (const void*)k_peel, kPeelDynSmem},
+    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_zorder", (const void*)k_zorder, 0}, {"k_peel", (const void*)k_peel, kPeelDynSmem},
                     {"k_stats", (const void*)k_stats, 0}, {"k_csr", (const void*)k_csr, 0},
                     {"k_niche", (const void*)k_niche, 0}, {"k_niche_oneshot", (const void*)k_niche_oneshot, 0},
                     {"k_peel_wave", (const void*)k_peel_wave, kPeelWaveDynSmem},

@@ -42,6 +42,13 @@ constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int64_t kMaxN2 = int64_t(1) << 21;
 constexpr int32_t kNotRanked = EMO_NOT_RANKED;
+// Ranking without a dominance matrix (k_fronts.cu) up to this many objectives:
+// with more, bounding boxes rule out too little (100,000 points of eight
+// objectives: 5.9 ms by the tree, 3.3 ms by the matrix; 40,000 of five: 0.20
+// and 0.26 ms).
+constexpr int kTreeMaxM = 5;
+constexpr int kTreeThreads = 1024;         // threads of its peeling kernel
+constexpr int kFrontLeafSmem = 64 * 1024;   // leaf states up to this size are copied to shared memory once per front
 
 enum Mode : int32_t { MODE_RANK = 1, MODE_SELECT = 2, MODE_HYPE = 3, MODE_DOM = 4 };
 
@@ -77,6 +84,17 @@ struct ProbIn {
     int64_t dom_ld;          // MODE_DOM: words per row
 };
 
+__forceinline__ __host__ __device__ bool tree_ranked(const ProbIn& in)
+{
+    return in.m <= kTreeMaxM && !in.ranked && in.mode != MODE_DOM;
+}
+// Whether the points are put in lexicographic order with prefix sets (the
+// dominance matrix, and the sample counts of TensorHypE).
+__forceinline__ __host__ __device__ bool lex_ordered(const ProbIn& in)
+{
+    return !in.ranked && (in.mode == MODE_DOM || in.mode == MODE_HYPE || !tree_ranked(in));
+}
+
 // Per-problem scalars; zeroed by the prep kernel.
 struct Scal {
     int32_t status;
@@ -101,7 +119,7 @@ struct Scal {
     float z[kMaxM];
     float inv_a32[kMaxM];
     double a[kMaxM];
-    unsigned int bar[2];     // barrier counters of the wide and the narrow groups (top bit: failed)
+    unsigned int bar[3];     // barrier counters of the narrow, wide and tree groups (top bit: failed)
     int32_t ncol;            // niching: keys collected from the selected histogram bin
     int32_t nsel;            // one-shot niching: references that took their nearest candidate
     int32_t longrun;         // sort: a run of equal f_1 longer than the in-place fix-up handles
@@ -154,6 +172,21 @@ struct ProbDev {
     unsigned char* colpre;   // [ncb][K] column-block prefix sets (colprep_obj_bytes each; K = m - 1 key
                              // objectives, or all m of the caller-order columns in MODE_DOM)
     float* ckeys;            // MODE_DOM: [n2p][m] objectives in caller order (padding -inf)
+    // ranking by the z-order tree (tree_ranked): points in grid-cell order,
+    // leaves of 32 points, nodes of 32 leaves, state of even and odd fronts
+    int32_t tree;
+    int32_t zbits, ncell;    // grid bits per objective, cells
+    int32_t nleaf, nnode, nleafp, nnodep;  // (p: rounded up to 32)
+    uint32_t* zcell;         // [n2] cell of each point (caller order)
+    uint32_t* zslot;         // [n2] its slot in the cell
+    uint32_t* zcnt;          // [ncell] cell counts, then offsets
+    float* zpts;             // [m][nleaf * 32] objectives in cell order
+    int32_t* zidx;           // [nleaf * 32] caller index
+    uint32_t* zkey;          // [nleaf * 32] cell
+    int32_t* zwit;           // [nleaf * 32] witness: an unranked dominator (-1: none known)
+    uint32_t* zlocal;        // [4 (nleafp + G)] bookkeeping of the leaves of large CTA shares
+    float* zstate;           // [2] minima of the nodes [m][nnodep] and of the leaves [m][nleafp] (unranked
+                             // points), and the leaves' masks of unranked points [nleafp]
     int32_t* spos;           // MODE_DOM: [2][n2] run of identical points of each caller index: first
                              // sorted position (-1 when alone), one past the last
 };
@@ -181,7 +214,8 @@ struct Plan {
     int32_t G;               // CTAs of every cooperative launch
     long long spin_budget;   // cycles a bounded wait may spin
     int32_t grp_first[kMaxBatch + 1];     // cooperative CTA groups of the peeling and TensorHypE kernels
-    int32_t grpn_first[kMaxBatch + 1];    // groups of the other cooperative kernels (at most as large)
+    int32_t grpn_first[kMaxBatch + 1];    // groups of the other cooperative kernels
+    int32_t grpt_first[kMaxBatch + 1];    // groups of the peeling by the z-order tree
     long long dom_item_start[kMaxBatch + 1];
     long long dom_items;
     unsigned long long dom_ctr[kMaxM + 1];  // dynamic work counters per objective count
@@ -254,6 +288,30 @@ __host__ __device__ constexpr int64_t colprep_obj_bytes(int K)
     return colprep_bkt_off(K) + (colprep_has_buckets(K) ? 128 + kPrefBuckets * 4 : 0);
 }
 
+// Bits per objective of the z-order grid: about one cell per half a point,
+// at most 2^18 cells (2^16 counters stay in L2 beside everything else) and 256
+// lines per objective.
+__host__ __device__ __forceinline__ int z_bits(int64_t n2, int m)
+{
+    int b = 1;
+    while ((int64_t(1) << b) < n2) ++b;
+    b = (b + 1 < 18 ? b + 1 : 18) / m;
+    return b < 1 ? 1 : (b > 8 ? 8 : b);
+}
+__host__ __device__ constexpr int64_t fronts_leaf_bytes(int64_t nleaf, int m) { return (nleaf + 31) / 32 * 32 * (m + 1) * 4; }
+// Leaves of one CTA that k_fronts keeps in its shared memory (witnesses and
+// objectives of 32 points each: 256 leaves of three objectives take 132 KB).
+__host__ __device__ constexpr int front_local(int m) { return m <= 3 ? 256 : 128; }
+// Dynamic shared memory of k_fronts for one problem: the nodes' state, the
+// leaves' when it is small, and the CTA's own leaves (witness, objectives and
+// four words of bookkeeping).
+__host__ __device__ __forceinline__ int fronts_smem_bytes(int64_t n2, int m)
+{
+    const int64_t nleaf = cdiv(n2, 32), nnode = cdiv(nleaf, 32), lb = fronts_leaf_bytes(nleaf, m);
+    return (int)((nnode + 31) / 32 * 32 * m * 4 + (lb <= kFrontLeafSmem ? lb : 0) +
+                 (nleaf < front_local(m) ? nleaf : front_local(m)) * (4 + 32 * (m + 1)) * 4);
+}
+
 // Byte layout of one problem region; fills `d` when base != 0. Returns the
 // region size. The same function sizes the workspace on the host and carves
 // it on the device.
@@ -261,22 +319,25 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
 {
     const int64_t n2 = in.n2, m = in.m, nr = (in.mode == MODE_SELECT || in.mode == MODE_HYPE) ? in.n_r : 1;
     const int64_t nrb = cdiv(n2, 32), ncb = cdiv(n2, kColBlock), n2p = ncb * kColBlock;
+    const bool tree = tree_ranked(in), lex = lex_ordered(in);
+    // (the tiles' space stays in the size that callers reserve, about n2^2 / 16
+    // bytes, also where the ranks come from the tree and nothing touches it)
     const int64_t ntiles = tiles_before(nrb, ncb);
     int64_t off = 0;
     auto take = [&](int64_t bytes) { int64_t o = off; off = align_up(off + bytes, 256); return o; };
     int64_t o_sc = take(sizeof(Scal));
-    int64_t o_idx = take(2 * n2p * 4);
-    int64_t o_keys = take(n2p * (m - 1) * 4);
-    int64_t o_runstart = take(n2p * 4);
-    int64_t o_minrs = take(ncb * 4);
-    int64_t o_cnt = take(n2p * 4);
+    int64_t o_idx = take(lex ? 2 * n2p * 4 : 0);
+    int64_t o_keys = take(lex ? n2p * (m - 1) * 4 : 0);
+    int64_t o_runstart = take(lex ? n2p * 4 : 0);
+    int64_t o_minrs = take(lex ? ncb * 4 : 0);
+    int64_t o_cnt = take(tree ? 0 : n2p * 4);
     int64_t o_rank_s = take(n2p * 4);
     int64_t o_rank_o = take(n2 * 4);
-    int64_t o_front = take(3 * n2p * 4);
-    int64_t o_front_n = take(3 * ncb * 4);
-    int64_t o_wdone = take(2 * ncb * 4);
-    int64_t o_wcnt = take((n2 + 2) * 4);
-    int64_t o_wofs = (in.ranked || in.mode == MODE_DOM) ? 0 : take(ncb * (n2 + 2) * 2);
+    int64_t o_front = take(tree ? 0 : 3 * n2p * 4);
+    int64_t o_front_n = take(tree ? 0 : 3 * ncb * 4);
+    int64_t o_wdone = take(tree ? 0 : 2 * ncb * 4);
+    int64_t o_wcnt = take(tree ? 0 : (n2 + 2) * 4);
+    int64_t o_wofs = (in.ranked || in.mode == MODE_DOM || tree) ? 0 : take(ncb * (n2 + 2) * 2);
     int64_t o_slist = take(n2 * 4);
     int64_t o_hist = take(int64_t(G) * kRadix * 4);
     int64_t o_flag = take((n2p + 1) * 4);
@@ -313,8 +374,24 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
     // the prefix sets, the dominance tiles and the wavefront offsets are not
     // needed when the ranks are given
     const int64_t kobj = in.mode == MODE_DOM ? m : m - 1;  // objectives with prefix sets
-    int64_t o_colpre = in.ranked ? 0 : take(ncb * kobj * colprep_obj_bytes((int)kobj));
+    int64_t o_colpre = lex ? take(ncb * kobj * colprep_obj_bytes((int)kobj)) : 0;
     int64_t o_D = (in.ranked || in.mode == MODE_DOM) ? 0 : take(ntiles * 4096);
+    // the z-order tree
+    const int64_t nleaf = cdiv(n2, 32), nnode = cdiv(nleaf, 32), nleafp = align_up(nleaf, 32), nnodep = align_up(nnode, 32);
+    const int64_t zb = z_bits(n2, (int)m), ncell = int64_t(1) << (zb * m), zs = nleaf * 32;
+    int64_t o_zcell = 0, o_zslot = 0, o_zcnt = 0, o_zpts = 0, o_zidx = 0, o_zkey = 0, o_zwit = 0, o_zlocal = 0,
+            o_zstate = 0;
+    if (tree) {
+        o_zcell = take(n2 * 4);
+        o_zslot = take(n2 * 4);
+        o_zcnt = take(ncell * 4);
+        o_zpts = take(m * zs * 4);
+        o_zidx = take(zs * 4);
+        o_zkey = take(zs * 4);
+        o_zwit = take(zs * 4);
+        o_zlocal = take(4 * (nleafp + G) * 4);
+        o_zstate = take(2 * (m * nnodep + (m + 1) * nleafp) * 4);
+    }
     int64_t o_ckeys = in.mode == MODE_DOM ? take(n2p * m * 4) : 0;
     int64_t o_spos = in.mode == MODE_DOM ? take(2 * n2 * 4) : 0;
     if (base && d) {
@@ -336,7 +413,7 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
         d->wdone = (int32_t*)(base + o_wdone);
         d->wmaxf = d->wdone + ncb;
         d->wcnt = (int32_t*)(base + o_wcnt);
-        d->wofs = (in.ranked || in.mode == MODE_DOM) ? nullptr : (uint16_t*)(base + o_wofs);
+        d->wofs = (in.ranked || in.mode == MODE_DOM || tree) ? nullptr : (uint16_t*)(base + o_wofs);
         d->slist = (int32_t*)(base + o_slist);
         d->hist = (int32_t*)(base + o_hist);
         d->flag = (int32_t*)(base + o_flag);
@@ -357,8 +434,24 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
         d->rphi2 = in.mode == MODE_SELECT ? (float*)(base + o_rphi2) : nullptr;
         d->rsort = in.mode == MODE_SELECT ? (float*)(base + o_rsort) : nullptr;
         d->flagged_bound = in.mode == MODE_SELECT ? (float*)(base + o_fbound) : nullptr;
-        d->colpre = in.ranked ? nullptr : (unsigned char*)(base + o_colpre);
+        d->colpre = lex ? (unsigned char*)(base + o_colpre) : nullptr;
         d->D = (in.ranked || in.mode == MODE_DOM) ? nullptr : (uint32_t*)(base + o_D);
+        d->tree = tree;
+        d->zbits = (int32_t)zb;
+        d->ncell = tree ? (int32_t)ncell : 0;
+        d->nleaf = (int32_t)nleaf;
+        d->nnode = (int32_t)nnode;
+        d->nleafp = (int32_t)nleafp;
+        d->nnodep = (int32_t)nnodep;
+        d->zcell = tree ? (uint32_t*)(base + o_zcell) : nullptr;
+        d->zslot = tree ? (uint32_t*)(base + o_zslot) : nullptr;
+        d->zcnt = tree ? (uint32_t*)(base + o_zcnt) : nullptr;
+        d->zpts = tree ? (float*)(base + o_zpts) : nullptr;
+        d->zidx = tree ? (int32_t*)(base + o_zidx) : nullptr;
+        d->zkey = tree ? (uint32_t*)(base + o_zkey) : nullptr;
+        d->zwit = tree ? (int32_t*)(base + o_zwit) : nullptr;
+        d->zlocal = tree ? (uint32_t*)(base + o_zlocal) : nullptr;
+        d->zstate = tree ? (float*)(base + o_zstate) : nullptr;
         d->ckeys = in.mode == MODE_DOM ? (float*)(base + o_ckeys) : nullptr;
         d->spos = in.mode == MODE_DOM ? (int32_t*)(base + o_spos) : nullptr;
     }
@@ -444,8 +537,7 @@ constexpr unsigned kBarFailed = 0x80000000u;
 __device__ __forceinline__ void set_status(Scal* sc, int code)
 {
     atomicCAS(&sc->status, 0, code);
-    atomicOr(&sc->bar[0], kBarFailed);
-    atomicOr(&sc->bar[1], kBarFailed);
+    for (unsigned& b : sc->bar) atomicOr(&b, kBarFailed);
 }
 
 // Group of CTAs serving one problem inside a cooperative launch.
@@ -455,20 +547,22 @@ struct Group {
     int size;       // CTAs in the group
     unsigned* bar;  // the group's barrier counter (all kernels of one assignment use the same size)
 };
-// The group of this CTA in the wide (peeling, TensorHypE) or the narrow
-// (every other cooperative kernel) assignment; prob = -1 for a CTA that
-// serves no problem (groups are capped by the problems' launch shapes), which
-// returns at once.
-__device__ __forceinline__ Group group_of(const Plan* plan, bool wide)
+// The group of this CTA in the wide (peeling from the matrix, TensorHypE),
+// the tree (peeling by the z-order tree) or the narrow (every other
+// cooperative kernel) assignment; prob = -1 for a CTA that serves no problem
+// (groups are capped by the problems' sizes and launch shapes), which returns
+// at once.
+enum GroupKind : int { GRP_NARROW = 0, GRP_WIDE = 1, GRP_TREE = 2 };
+__device__ __forceinline__ Group group_of(const Plan* plan, GroupKind kind)
 {
-    const int32_t* first = wide ? plan->grp_first : plan->grpn_first;
+    const int32_t* first = kind == GRP_WIDE ? plan->grp_first : (kind == GRP_TREE ? plan->grpt_first : plan->grpn_first);
     Group g;
     int b = blockIdx.x, p = 0;
     while (p + 1 < plan->nprob && first[p + 1] <= b) ++p;
     g.prob = b < first[plan->nprob] ? p : -1;
     g.rank = b - first[p];
     g.size = first[p + 1] - first[p];
-    g.bar = &plan->p[p].sc->bar[wide ? 0 : 1];
+    g.bar = &plan->p[p].sc->bar[kind];
     return g;
 }
 

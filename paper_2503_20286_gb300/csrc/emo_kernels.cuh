@@ -205,6 +205,8 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws);
 __global__ void k_prep(Plan* plan);
 __global__ void k_sort(Plan* plan);
 __global__ void k_peel(Plan* plan);
+__global__ void k_zorder(Plan* plan);
+__global__ void k_fronts(Plan* plan);
 
 constexpr int kPeelChunk = 8192;   // front members staged in shared memory at once
 constexpr int kPeelStages = 2;     // per-warp ring of 32-row copies (one batch in flight while one is counted)

@@ -10,7 +10,8 @@
 //     The set {q in half : f_k(q) >= f_k(p)} is then a prefix of that order:
 //     a checkpoint bitset plus at most CPS - 1 extra bits (CPS = 1 for m <= 4,
 //     so no extra bits at all).
-//   k_dom_pref<M> (m <= 6; k_dom_pref_rt for m >= 7) -- one warp per row
+//   k_dom_pref<M> (m = 6; k_dom_pref_rt for m >= 7; up to five objectives are
+//     ranked without the matrix, k_fronts.cu) -- one warp per row
 //     block: each lane first counts, for its row and each objective, the
 //     columns of both halves that are >= (binary search). Then each half-warp
 //     builds one row at a time (lanes 0-15 rows 0-15, lanes 16-31 rows 16-31),
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
         for (int p = pfirst; p < plast; ++p) {
             s_first[p - pfirst] = acc;
             const ProbDev& d = plan->p[p];
-            if (ld_volatile(&d.sc->status) == 0) acc += (long long)d.ncb * keys_of(d);
+            if (d.colpre && ld_volatile(&d.sc->status) == 0) acc += (long long)d.ncb * keys_of(d);
         }
         s_first[plast - pfirst] = acc;
     }
@@ -280,19 +281,11 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
 }
 
 // ------------------------------------------------------------ k_dom_pref
-// Objectives whose prefix sets have a checkpoint at every count and room in
-// shared memory (at most two keys): the rows' checkpoint offsets are staged
-// per warp in shared memory instead of being broadcast by shuffles.
-template <int K>
-constexpr bool kStageOffsets = K <= 2 && PrefShape<K>::LOG_CPS == 0;
-
 template <int K>
 struct PrefSmem {
     alignas(128) unsigned char obj[K * PrefShape<K>::OBJ_BYTES];
     alignas(128) int32_t rs[kColBlock];
     int32_t cnt[kColBlock];
-    // per warp, objective and half: byte offset t * 128 of each row's checkpoint
-    uint32_t off[kStageOffsets<K> ? 16 * K * 64 : 1];
     uint64_t bar;
     long long item;
     int skip;
@@ -408,41 +401,6 @@ __device__ __forceinline__ void pref_rows(const unsigned char* __restrict__ obj,
                 word &= prefix_word<S::LOG_CPS, S::ORD_OFF>(obj + k * S::OBJ_BYTES, tk, l);
             }
             word = row_masks<DIAG, DUP>(word, rowbase + i, cbase, rs, l);
-            __stcs(dst + j * 16, word);
-            xl[jj] = (uint32_t)word;
-            xh[jj] = (uint32_t)(word >> 32);
-        }
-        vlo.add8_warp(xl);
-        vhi.add8_warp(xh);
-    }
-}
-
-// pref_rows with the rows' checkpoint offsets read from this warp's staged
-// offsets `so` ([K][2 halves][32 rows], bytes t * 128 of the half's count):
-// one shared load per row and objective replaces a shuffle, a byte permute
-// and the offset arithmetic.
-template <int K, bool DIAG, bool DUP>
-__device__ __forceinline__ void pref_rows_off(const unsigned char* __restrict__ obj,
-                                              const int32_t* __restrict__ rs, const uint32_t* so, int64_t rowbase,
-                                              int64_t cbase, uint32_t* tile, VCount<kDomNH>& vlo,
-                                              VCount<kDomNH>& vhi, int lane)
-{
-    using S = PrefShape<K>;
-    const int l = lane & 15, h = lane >> 4;
-    const uint32_t* my = so + (l >> 3) * 32 + 16 * h;  // this lane's half; rows j + 16 h
-    const unsigned char* pb = obj + kPrefPbOff + l * 8;
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(tile + h * 16 * 32) + l;
-#pragma unroll 1
-    for (int g = 0; g < 2; ++g) {
-        uint32_t xl[8], xh[8];
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            const int j = g * 8 + jj;
-            unsigned long long word = ~0ull;
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                word &= *reinterpret_cast<const unsigned long long*>(pb + k * S::OBJ_BYTES + my[k * 64 + j]);
-            word = row_masks<DIAG, DUP>(word, rowbase + j + 16 * h, cbase, rs, l);
             __stcs(dst + j * 16, word);
             xl[jj] = (uint32_t)word;
             xh[jj] = (uint32_t)(word >> 32);
@@ -571,23 +529,9 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
             const bool dup = rb * kTileRows + 31 >= dupcut;
             const int64_t rowbase = (int64_t)rb * kTileRows;
             uint32_t* tile = Dm + tile_index(rb, cb, ncb) * (int64_t)(kTileRows * kTileWords);
-            if constexpr (kStageOffsets<K>) {
-                uint32_t* so = sm.off + warp * (K * 64);
-                __syncwarp();  // the previous row block's offsets have been read
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    so[k * 64 + lane] = (uint32_t)(t[k] & 0xffff) * 128u;
-                    so[k * 64 + 32 + lane] = (uint32_t)(t[k] >> 16) * 128u;
-                }
-                __syncwarp();
-                if (dup) pref_rows_off<K, true, true>(sm.obj, sm.rs, so, rowbase, cbase, tile, vlo, vhi, lane);
-                else if (diag) pref_rows_off<K, true, false>(sm.obj, sm.rs, so, rowbase, cbase, tile, vlo, vhi, lane);
-                else pref_rows_off<K, false, false>(sm.obj, sm.rs, so, rowbase, cbase, tile, vlo, vhi, lane);
-            } else {
-                if (dup) pref_rows<K, true, true>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
-                else if (diag) pref_rows<K, true, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
-                else pref_rows<K, false, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
-            }
+            if (dup) pref_rows<K, true, true>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
+            else if (diag) pref_rows<K, true, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
+            else pref_rows<K, false, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
         }
         dom_flush_item(d, cbase, vlo, vhi, sm.cnt, lane);
     }
@@ -1073,13 +1017,9 @@ cudaError_t launch_dominance_tri_range(int m, Plan* plan, int sms, cudaStream_t 
     (void)pfirst;
     (void)plast;
     switch (m) {
-    case 2: return launch_tri_m<2>(plan, sms, s, lo, hi, counter);
-    case 3: return launch_tri_m<3>(plan, sms, s, lo, hi, counter);
-    case 4: return launch_tri_m<4>(plan, sms, s, lo, hi, counter);
-    case 5: return launch_tri_m<5>(plan, sms, s, lo, hi, counter);
     case 6: return launch_tri_m<6>(plan, sms, s, lo, hi, counter);
     default:
-        if (m < 2 || m > kMaxM) return cudaErrorInvalidValue;
+        if (m <= kTreeMaxM || m > kMaxM) return cudaErrorInvalidValue;  // (fewer objectives need no matrix)
         return launch_tri_rt(m - 1, plan, sms, s, lo, hi, counter);
     }
 }

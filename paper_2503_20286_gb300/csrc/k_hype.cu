@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_hype(Plan* plan, int phase)
     __shared__ __align__(16) float s_pts[kHypeTile];
     __shared__ RadixSmem rsm;
     __shared__ uint32_t s_key[kMaxM];
-    const Group g = group_of(plan, true);
+    const Group g = group_of(plan, GRP_WIDE);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;

@@ -19,7 +19,7 @@ namespace emo {
 // ------------------------------------------------------------ k_csr
 __global__ void __launch_bounds__(kCoopThreads, 1) k_csr(Plan* plan)
 {
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
@@ -570,7 +570,7 @@ __device__ bool niche_bulk(const ProbDev& d, const Group& g, long long budget, i
 __global__ void __launch_bounds__(kCoopThreads, 1) k_niche(Plan* plan)
 {
     __shared__ NicheSmem sm;
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
@@ -693,7 +693,7 @@ __device__ __forceinline__ unsigned long long oneshot_key(uint64_t seed, uint64_
 __global__ void __launch_bounds__(kCoopThreads, 1) k_niche_oneshot(Plan* plan)
 {
     __shared__ NicheSmem sm;
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
@@ -776,7 +776,7 @@ cudaError_t sticky_merge(const int32_t* status, cudaStream_t s)
 // and the optional intermediates.
 __global__ void __launch_bounds__(kCoopThreads, 1) k_finish(Plan* plan)
 {
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;

@@ -120,12 +120,12 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
     // [ring] per-warp copy stages | [ncb + 1] member prefix per block | [kPeelChunk] staged members
     extern __shared__ __align__(128) int s_dyn[];
 
-    const Group g = group_of(plan, true);
+    const Group g = group_of(plan, GRP_WIDE);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
     const long long budget = plan->spin_budget;
-    if (ld_volatile(&d.sc->status) != 0) return;
+    if (d.tree || ld_volatile(&d.sc->status) != 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n2 = in.n2, n2p = d.n2p;
     const int ncb = d.ncb;
@@ -404,12 +404,12 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel_wave(Plan* plan)
     // [ncb] owned blocks | [ncb] next front of each owned block (kInf: finished)
     extern __shared__ __align__(128) int s_dyn[];
 
-    const Group g = group_of(plan, true);
+    const Group g = group_of(plan, GRP_WIDE);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
     const long long budget = plan->spin_budget;
-    if (ld_volatile(&d.sc->status) != 0) return;
+    if (d.tree || ld_volatile(&d.sc->status) != 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n2 = in.n2;
     const int ncb = d.ncb;

@@ -22,11 +22,61 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
         ProbDev d;
         layout_problem(a.in[t], a.G, ws + a.in[t].ws_off, &d);
         plan->p[t] = d;
-        char* sc = (char*)d.sc;
-        for (size_t i = 0; i < sizeof(Scal); ++i) sc[i] = 0;
     }
-    __syncthreads();
-    if (t == 0) {
+    for (int p = t >> 5; p < a.nprob; p += blockDim.x >> 5) {  // (the scalars open the region)
+        uint32_t* sc = reinterpret_cast<uint32_t*>(ws + a.in[p].ws_off);
+        for (int i = t & 31; i < (int)(sizeof(Scal) / 4); i += 32) sc[i] = 0u;
+    }
+    // CTA groups of each kind: shares of the grid in proportion to the work,
+    // at least one CTA for every problem that the kind serves and at most the
+    // problem's cap. Wide groups by n2^2 (dominance tiles read per front), tree
+    // groups by the searches to expect, narrow ones by n2. CTAs beyond the groups serve no problem.
+    if (t < 96 && (t & 31) == 0) {
+        const GroupKind kind = (GroupKind)(t >> 5);
+        auto weight = [&](int p) -> double {
+            const ProbIn& in = a.in[p];
+            const double n = (double)in.n2;
+            if (kind == GRP_WIDE) return tree_ranked(in) && in.mode != MODE_HYPE ? 0.0 : n * n;
+            // (searches grow with m: 5 ms of CTA time for 20,000 points of three
+            // objectives, 16 ms for 40,000 of five)
+            if (kind == GRP_TREE) return tree_ranked(in) ? n * (in.m - 1) : 0.0;
+            return n;
+        };
+        auto cap = [&](int p) -> int {
+            const ProbIn& in = a.in[p];
+            int c = in.cap_wide > 0 ? min(in.cap_wide, a.G) : a.G;
+            if (kind == GRP_NARROW && in.cap_narrow > 0) c = min(c, in.cap_narrow);
+            if (kind == GRP_TREE) c = min(c, (int)max((int64_t)1, cdiv(cdiv(in.n2, 32), kTreeThreads / 64)));
+            return c;
+        };
+        int32_t* first = kind == GRP_WIDE ? plan->grp_first : (kind == GRP_TREE ? plan->grpt_first : plan->grpn_first);
+        double tot = 0.0;
+        int served = 0;
+        for (int p = 0; p < a.nprob; ++p) {
+            const double w = weight(p);
+            tot += w;
+            served += w > 0.0;
+        }
+        const double per = tot > 0.0 ? (double)(a.G - served) / tot : 0.0;
+        int cnt[kMaxBatch], given = 0;
+        for (int p = 0; p < a.nprob; ++p) {
+            const double w = weight(p);
+            cnt[p] = w > 0.0 ? min(cap(p), 1 + (int)(w * per)) : 0;
+            given += cnt[p];
+        }
+        for (bool grew = true; given < a.G && grew;) {
+            grew = false;
+            for (int p = 0; p < a.nprob && given < a.G; ++p)
+                if (cnt[p] > 0 && cnt[p] < cap(p)) { cnt[p]++; given++; grew = true; }
+        }
+        int acc = 0;
+        for (int p = 0; p < a.nprob; ++p) {
+            first[p] = acc;
+            acc += cnt[p];
+        }
+        first[a.nprob] = acc;
+    }
+    if (t == 96) {
         plan->nprob = a.nprob;
         plan->G = a.G;
         plan->spin_budget = a.spin_budget;
@@ -34,39 +84,10 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
         for (int i = 0; i <= kMaxM; ++i) plan->dom_ctr[i] = 0;
         for (int i = 0; i <= kMaxM; ++i) plan->asc_next[i] = 0;
         plan->status = 0;
-        // Wide CTA groups (peeling, TensorHypE) proportional to n2^2 (the
-        // dominance and peeling work), at least one CTA each and at most the
-        // problem's cap_wide; narrow groups (the other cooperative kernels)
-        // the first min(wide, cap_narrow) CTAs' worth. CTAs beyond the
-        // groups serve no problem.
-        double tot = 0.0;
-        for (int p = 0; p < a.nprob; ++p) tot += (double)a.in[p].n2 * (double)a.in[p].n2;
-        int extra = a.G - a.nprob, given = 0;
-        int cnt[kMaxBatch];
-        auto cap_of = [&](int p, int32_t c) { return c > 0 ? c : a.G; };
-        for (int p = 0; p < a.nprob; ++p) {
-            double w = (double)a.in[p].n2 * (double)a.in[p].n2 / tot;
-            cnt[p] = min(cap_of(p, a.in[p].cap_wide), 1 + (int)(w * extra));
-            given += cnt[p];
-        }
-        for (bool grew = true; given < a.G && grew;) {
-            grew = false;
-            for (int p = 0; p < a.nprob && given < a.G; ++p)
-                if (cnt[p] < cap_of(p, a.in[p].cap_wide)) { cnt[p]++; given++; grew = true; }
-        }
-        int acc = 0, accn = 0;
-        for (int p = 0; p < a.nprob; ++p) {
-            plan->grp_first[p] = acc;
-            acc += cnt[p];
-            plan->grpn_first[p] = accn;
-            accn += min(cnt[p], cap_of(p, a.in[p].cap_narrow));
-        }
-        plan->grp_first[a.nprob] = acc;
-        plan->grpn_first[a.nprob] = accn;
         long long di = 0;
         for (int p = 0; p < a.nprob; ++p) {
             plan->dom_item_start[p] = di;
-            di += dom_items_of(a.in[p].n2, a.in[p].dom_chunk);
+            if (!tree_ranked(a.in[p])) di += dom_items_of(a.in[p].n2, a.in[p].dom_chunk);
         }
         plan->dom_item_start[a.nprob] = di;
         plan->dom_items = di;
@@ -115,15 +136,19 @@ __global__ void k_prep(Plan* plan)
         }
     }
     for (int64_t s = tid; s < d.n2p; s += stride) {
-        d.idx[s] = (int32_t)s;
-        d.cnt[s] = 0;
+        if (lex_ordered(in)) d.idx[s] = (int32_t)s;
+        if (!d.tree) d.cnt[s] = 0;
         d.rank_s[s] = kNotRanked;
         d.flag[s] = 0;
     }
+    for (int64_t c = tid; c < d.ncell; c += stride) d.zcnt[c] = 0u;
     for (int64_t i = tid; i < n2; i += stride) d.rank_o[i] = kNotRanked;
-    for (int64_t c = tid; c < 3 * (int64_t)d.ncb; c += stride) d.front_n[c] = 0;
-    for (int64_t c = tid; c < n2 + 2; c += stride) d.wcnt[c] = 0;  // front sizes of the wavefront peeling
-    for (int64_t c = tid; c < d.ncb; c += stride) d.minrs[c] = INT32_MAX;
+    if (!d.tree) {
+        for (int64_t c = tid; c < 3 * (int64_t)d.ncb; c += stride) d.front_n[c] = 0;
+        for (int64_t c = tid; c < n2 + 2; c += stride) d.wcnt[c] = 0;  // front sizes of the wavefront peeling
+    }
+    if (lex_ordered(in))
+        for (int64_t c = tid; c < d.ncb; c += stride) d.minrs[c] = INT32_MAX;
     if (in.mode == MODE_SELECT && !in.R) {
         for (int64_t j = tid; j < in.n_r; j += stride) {
             d.rho[j] = 0;
@@ -181,7 +206,7 @@ __device__ void sort_references(const ProbDev& d, const Group& g, long long budg
 // Lexicographic order, sorted objective keys and runs of equal points.
 __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
 {
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
@@ -192,7 +217,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
     const int gs = (int)max((int64_t)1, min((int64_t)g.size, cdiv(n2, 4096)));
     const float* F = in.F;
     __shared__ RadixSmem rsm;
-    if (in.ranked) {  // selection from given ranks: no dominance matrix, so no point order
+    if (!lex_ordered(in)) {  // ranks given, or ranked by the z-order tree: no lexicographic order of the points
         if (in.mode == MODE_SELECT) sort_references(d, g, budget, rsm);
         return;
     }

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_rank_in(Plan* plan)
 {
     __shared__ int s_warp[33];
     __shared__ int s_l, s_np, s_nl;
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_rank_in(Plan* plan)
 // range, then the niche counts of the range's points of P.
 __global__ void __launch_bounds__(kCoopThreads, 1) k_assoc_out(Plan* plan)
 {
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const SplitArgs& sp = plan->split;
     const ProbDev& d = plan->p[g.prob];
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_assoc_out(Plan* plan)
 // ascending caller order, each of rank l, |L| of them (so exactly front l).
 __global__ void __launch_bounds__(kCoopThreads, 1) k_given_in(Plan* plan)
 {
-    const Group g = group_of(plan, false);
+    const Group g = group_of(plan, GRP_NARROW);
     if (g.prob < 0) return;  // a CTA beyond every problem's group
     const SplitArgs& sp = plan->split;
     const ProbDev& d = plan->p[g.prob];
