@@ -118,7 +118,7 @@ DevInfo dev_info()
         const void* kernels[] = {(const void*)k_sort,  (const void*)k_peel,  (const void*)k_peel_wave,
                                  (const void*)k_stats, (const void*)k_csr,   (const void*)k_niche,
                                  (const void*)k_niche_oneshot, (const void*)k_hype, (const void*)k_finish,
-                                 (const void*)k_rank_in, (const void*)k_assoc_out, (const void*)k_given_in, (const void*)k_zorder,
+                                 (const void*)k_rank_in, (const void*)k_assoc_out, (const void*)k_given_in, (const void*)k_order,
                                  (const void*)k_fronts};
         const int dyn[] = {0, kPeelDynSmem, kPeelWaveDynSmem, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, kFrontsDynSmem};
         for (int i = 0; i < (int)(sizeof(dyn) / sizeof(dyn[0])); ++i) {
@@ -275,7 +275,9 @@ emo_status run_selection_stages(std::vector<ProbIn>& ins, const DevInfo& di, Pla
     const int bps = shape_for(dev, di.sms, ins[big].m, ins[big].n2).assoc_bps;
     if (launch_assoc(plan, nprob, m_of.data(), di.sms, bps, s) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("assoc");
-    k_rescan<<<di.sms * 2, 256, 0, s>>>(plan);
+    // (a grid row per problem, as many CTAs as the largest needs)
+    k_decide<<<dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(ins[big].n2, 256), di.sms * 8 / nprob)), nprob), 256,
+               0, s>>>(plan);
     if (cudaGetLastError() != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("rescan");
     if (split == SPLIT_ASSOC) {
@@ -367,9 +369,9 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     sm.mark("prep");
     // (from given ranks only the references are ordered; the niching from a
     // given association has none)
-    if (sp.kind != SPLIT_NICHE && (any_lex || any_select) && coop((const void*)k_sort, di.G, 0, s, plan) != cudaSuccess)
+    if (any_lex && coop((const void*)k_sort, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (sp.kind != SPLIT_NICHE && (any_tree || any_select) && coop((const void*)k_order, di.G, 0, s, plan) != cudaSuccess)
         return EMO_ERR_CUDA;
-    if (any_tree && coop((const void*)k_zorder, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("sort");
     if (nprob == 1 && ins[0].mode == MODE_DOM) {  // caller-order dominance matrix only
         const ProbIn& in = ins[0];
@@ -1063,7 +1065,7 @@ int32_t emo_device_report(char* buf, int32_t len)
     out += "; sms " + std::to_string(sms) + "; cooperative " + std::to_string(coop);
     DevInfo di = dev_info();  // also sets the dynamic shared memory limit of k_peel
     struct K { const char* name; const void* fn; int dyn; };
-    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_zorder", (const void*)k_zorder, 0}, {"k_peel", (const void*)k_peel, kPeelDynSmem},
+    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_order", (const void*)k_order, 0}, {"k_peel", (const void*)k_peel, kPeelDynSmem},
                     {"k_stats", (const void*)k_stats, 0}, {"k_csr", (const void*)k_csr, 0},
                     {"k_niche", (const void*)k_niche, 0}, {"k_niche_oneshot", (const void*)k_niche_oneshot, 0},
                     {"k_peel_wave", (const void*)k_peel_wave, kPeelWaveDynSmem},

@@ -103,19 +103,19 @@ struct Scal {
     int32_t ranked;          // points ranked so far
     int32_t nfronts;
     int32_t fallback;
-    int32_t nflag;           // points needing the all-reference FP64 scan
+    int32_t nflag;           // points associated by an FP64 scan of more than two references
     int32_t levels;
     int32_t front_total[2];  // members of the current / next front
     int32_t idx_buf;         // idx half holding the sorted order
     int32_t lbuf;            // llist half holding the sorted candidate lists
-    int32_t rbuf;            // rord half holding the angle order
+    int32_t nbad;            // points listed for the scan of every reference
     uint32_t zkey[kMaxM];
     uint32_t kor[kMaxM];     // OR of the order-preserving keys of each objective over all points
     uint32_t kinv[kMaxM];    // OR of their complements (a bit varies iff set in both)
     uint32_t asf32[kMaxM];
     unsigned long long asf64[kMaxM];
     int32_t ext[kMaxM];
-    unsigned long long nadir[kMaxM];
+    uint32_t fkey[kMaxM];    // largest order-preserving key of each objective over S
     float z[kMaxM];
     float inv_a32[kMaxM];
     double a[kMaxM];
@@ -126,6 +126,8 @@ struct Scal {
     int32_t lfinal1;         // wavefront peeling: l + 1 once known, 0 before
     unsigned long long rho_sum;  // niching from a given association: sum of the given niche counts
 };
+
+struct DirGrid;  // grid of the directions (cell_order.cuh)
 
 // Device-side descriptor with every workspace pointer of one problem.
 struct ProbDev {
@@ -153,12 +155,24 @@ struct ProbDev {
     int32_t* pi;             // [n2] associated reference
     double* d64;             // [n2] perpendicular distance (FP64)
     float* rhat;             // [n_r][m] unit reference directions (FP32)
-    int32_t* rord;           // [2][n_r] references sorted by polar angle from axis 1 (ping-pong)
-    float* rphi;             // [n_r] sorted polar angles (from axis 1)
-    float* rphi2;            // [n_r] angles from axis 2, in the same order
-    float* rsort;            // [n_r][m] unit directions in polar-angle order
-    int32_t* flagged;        // [n2] points for the exhaustive FP64 scan
-    float* flagged_bound;    // [n2] angular half-width of that scan (inf = all references)
+    // references in grid-cell order, leaves of 32, nodes of 32 leaves (k_order.cu)
+    int32_t rtree;           // MODE_SELECT with references
+    int32_t rbits, nrcell;   // grid bits per coordinate, cells
+    int32_t nrleaf, nrnode, nrleafp, nrnodep;  // (p: rounded up to 32)
+    DirGrid* rgrid;          // the references' grid
+    uint32_t* rcnt;          // [2][nrcell] cell counts, then offsets: references | S
+    uint32_t* rcell;         // [n_r] cell of each reference
+    uint32_t* rslot;         // [n_r] its slot in the cell
+    int32_t* rord;           // [n_r] sorted position -> reference
+    float* rsort;            // [nrleaf * 32][m rounded up to 4] unit directions in that order
+    float* rball;            // [m][nrleafp] mean direction of each leaf
+    float* rrad;             // [nrleafp] largest distance of a member from it
+    float* rnball;           // [m][nrnodep] the same of each node
+    float* rnrad;            // [nrnodep]
+    int32_t* sord;           // [n2] S in the order of the references' grid cells
+    uint32_t* scell;         // [n2] cell of each entry of slist
+    uint32_t* sslot;         // [n2] its slot in the cell
+    int32_t* flagged;        // [n2] points for the scan of every reference in FP64
     int32_t* rho;            // [n_r] niche counts of P (evolving during niching)
     int32_t* lcnt;           // [n_r] last-front members per reference (evolving)
     int32_t* loff;           // [n_r + 1] CSR offsets of the candidate lists
@@ -288,15 +302,23 @@ __host__ __device__ constexpr int64_t colprep_obj_bytes(int K)
     return colprep_bkt_off(K) + (colprep_has_buckets(K) ? 128 + kPrefBuckets * 4 : 0);
 }
 
-// Bits per objective of the z-order grid: about one cell per half a point,
-// at most 2^18 cells (2^16 counters stay in L2 beside everything else) and 256
-// lines per objective.
+// Bits per coordinate of a z-order grid over n items: about two cells per
+// item, at most 2^18 cells (1 MB of counters) and 256 lines per coordinate.
 __host__ __device__ __forceinline__ int z_bits(int64_t n2, int m)
 {
     int b = 1;
     while ((int64_t(1) << b) < n2) ++b;
     b = (b + 1 < 18 ? b + 1 : 18) / m;
     return b < 1 ? 1 : (b > 8 ? 8 : b);
+}
+// Bits per coordinate of the directions' grid: about four cells per reference,
+// at most 2^18.
+__host__ __device__ __forceinline__ int dir_bits(int64_t nr, int dims)
+{
+    int b = 1;
+    while ((int64_t(1) << b) < nr) ++b;
+    b = (b + 2 < 18 ? b + 2 : 18) / dims;
+    return b < 1 ? 1 : b;
 }
 __host__ __device__ constexpr int64_t fronts_leaf_bytes(int64_t nleaf, int m) { return (nleaf + 31) / 32 * 32 * (m + 1) * 4; }
 // Leaves of one CTA that k_fronts keeps in its shared memory (witnesses and
@@ -342,8 +364,12 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
     int64_t o_hist = take(int64_t(G) * kRadix * 4);
     int64_t o_flag = take((n2p + 1) * 4);
     int64_t o_pi = 0, o_d64 = 0, o_rhat = 0, o_flagged = 0, o_rho = 0, o_lcnt = 0, o_loff = 0,
-            o_llist = 0, o_fen = 0, o_ekeys = 0, o_elist = 0, o_rord = 0, o_rphi = 0, o_rsort = 0, o_fbound = 0,
-            o_nhist = 0, o_rphi2 = 0;
+            o_llist = 0, o_fen = 0, o_ekeys = 0, o_elist = 0, o_rord = 0, o_rsort = 0, o_nhist = 0, o_rgrid = 0,
+            o_rcnt = 0, o_rcell = 0, o_rslot = 0, o_rball = 0, o_rrad = 0, o_rnball = 0, o_rnrad = 0, o_sord = 0,
+            o_scell = 0, o_sslot = 0;
+    const int64_t nrleaf = cdiv(nr, 32), nrnode = cdiv(nrleaf, 32), nrleafp = align_up(nrleaf, 32),
+                  nrnodep = align_up(nrnode, 32), rdims = m <= 3 ? m - 1 : m, rbits = dir_bits(nr, (int)rdims),
+                  nrcell = int64_t(1) << (rbits * rdims);
     if (in.mode == MODE_SELECT) {
         o_pi = take(n2 * 4);
         o_d64 = take(n2 * 8);
@@ -356,11 +382,19 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
         o_fen = take(n2 * 4);
         o_ekeys = take((nr > n2 ? nr : n2) * 8);
         o_elist = take(nr * 4);
-        o_rord = take(2 * nr * 4);
-        o_rphi = take(nr * 4);
-        o_rphi2 = take(nr * 4);
-        o_rsort = take(nr * m * 4);
-        o_fbound = take(n2 * 4);
+        o_rord = take(nr * 4);
+        o_rsort = take(nrleaf * 32 * align_up(m, 4) * 4);
+        o_rgrid = take(2 * kMaxM * 4);
+        o_rcnt = take(2 * nrcell * 4);
+        o_rcell = take(nr * 4);
+        o_rslot = take(nr * 4);
+        o_rball = take(m * nrleafp * 4);
+        o_rrad = take(nrleafp * 4);
+        o_rnball = take(m * nrnodep * 4);
+        o_rnrad = take(nrnodep * 4);
+        o_sord = take(n2 * 4);
+        o_scell = take(n2 * 4);
+        o_sslot = take(n2 * 4);
         o_nhist = take(kNicheBins * 4 + int64_t(G) * 8);
     } else if (in.mode == MODE_HYPE) {
         // d64: contributions; rhat: samples; rho: their dominator counts;
@@ -430,10 +464,26 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
         d->elist = in.mode == MODE_SELECT ? (int32_t*)(base + o_elist) : nullptr;
         d->nhist = in.mode == MODE_SELECT ? (int32_t*)(base + o_nhist) : nullptr;
         d->rord = in.mode == MODE_SELECT ? (int32_t*)(base + o_rord) : nullptr;
-        d->rphi = in.mode == MODE_SELECT ? (float*)(base + o_rphi) : nullptr;
-        d->rphi2 = in.mode == MODE_SELECT ? (float*)(base + o_rphi2) : nullptr;
         d->rsort = in.mode == MODE_SELECT ? (float*)(base + o_rsort) : nullptr;
-        d->flagged_bound = in.mode == MODE_SELECT ? (float*)(base + o_fbound) : nullptr;
+        const bool rt = in.mode == MODE_SELECT;
+        d->rtree = rt && in.R;
+        d->rbits = (int32_t)rbits;
+        d->nrcell = rt ? (int32_t)nrcell : 0;
+        d->nrleaf = (int32_t)nrleaf;
+        d->nrnode = (int32_t)nrnode;
+        d->nrleafp = (int32_t)nrleafp;
+        d->nrnodep = (int32_t)nrnodep;
+        d->rgrid = rt ? (DirGrid*)(base + o_rgrid) : nullptr;
+        d->rcnt = rt ? (uint32_t*)(base + o_rcnt) : nullptr;
+        d->rcell = rt ? (uint32_t*)(base + o_rcell) : nullptr;
+        d->rslot = rt ? (uint32_t*)(base + o_rslot) : nullptr;
+        d->rball = rt ? (float*)(base + o_rball) : nullptr;
+        d->rrad = rt ? (float*)(base + o_rrad) : nullptr;
+        d->rnball = rt ? (float*)(base + o_rnball) : nullptr;
+        d->rnrad = rt ? (float*)(base + o_rnrad) : nullptr;
+        d->sord = rt ? (int32_t*)(base + o_sord) : nullptr;
+        d->scell = rt ? (uint32_t*)(base + o_scell) : nullptr;
+        d->sslot = rt ? (uint32_t*)(base + o_sslot) : nullptr;
         d->colpre = lex ? (unsigned char*)(base + o_colpre) : nullptr;
         d->D = (in.ranked || in.mode == MODE_DOM) ? nullptr : (uint32_t*)(base + o_D);
         d->tree = tree;
@@ -626,23 +676,6 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
     }
     return c;
 }
-// Polar angle of a direction from objective axis 1, atan2(|v_2..m|, v_1):
-// well conditioned everywhere (unlike acos of a cosine near 0).
-__device__ __forceinline__ float polar_angle(const float* v, int m)
-{
-    float s = 0.0f;
-    for (int k = 1; k < m; ++k) s = fmaf(v[k], v[k], s);
-    return atan2f(sqrtf(s), v[0]);
-}
-// Angle from axis 2, by the same formula (the second pivot of the association
-// index).
-__device__ __forceinline__ float polar_angle2(const float* v, int m)
-{
-    float s = v[0] * v[0];
-    for (int k = 2; k < m; ++k) s = fmaf(v[k], v[k], s);
-    return atan2f(sqrtf(s), v[1]);
-}
-
 // Niching stream: key = seed, counter = (j, 2 c + tag, generation).
 __device__ __forceinline__ uint32_t niche_random(uint64_t seed, uint64_t gen, uint32_t j, uint32_t c, uint32_t tag)
 {

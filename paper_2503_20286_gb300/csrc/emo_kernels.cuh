@@ -205,7 +205,7 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws);
 __global__ void k_prep(Plan* plan);
 __global__ void k_sort(Plan* plan);
 __global__ void k_peel(Plan* plan);
-__global__ void k_zorder(Plan* plan);
+__global__ void k_order(Plan* plan);
 __global__ void k_fronts(Plan* plan);
 
 constexpr int kPeelChunk = 8192;   // front members staged in shared memory at once
@@ -225,7 +225,7 @@ cudaError_t launch_front_counts(const uint32_t* D, int64_t ld, int64_t ncols, co
                                 int32_t* counts, uint8_t* new_front, int sms, cudaStream_t s);
 __host__ __device__ constexpr int peel_wave_smem_bytes(int ncb) { return peel_smem_bytes(ncb) + 2 * ncb * (int)sizeof(int); }
 __global__ void k_stats(Plan* plan);
-__global__ void k_rescan(Plan* plan);
+__global__ void k_decide(Plan* plan);
 __global__ void k_csr(Plan* plan);
 __global__ void k_niche(Plan* plan);
 __global__ void k_niche_oneshot(Plan* plan);

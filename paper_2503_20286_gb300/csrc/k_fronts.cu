@@ -8,7 +8,7 @@
 // witness) is known, and a new witness is sought only when the old one has
 // been ranked -- about two searches per point in all. A search is a walk over a
 // two-level tree of bounding boxes:
-//   * k_zorder puts the points in the order of the Morton (z-order) cells of a
+//   * k_order puts the points in the order of the Morton (z-order) cells of a
 //     grid whose lines are sample quantiles of each objective. 32 consecutive
 //     points form a leaf, 32 leaves a node. Dominance never points backwards
 //     along this order (p <= q in every objective puts p's cell no later).
@@ -38,125 +38,6 @@
 #include "emo_kernels.cuh"
 
 namespace emo {
-
-constexpr int kZSample = 512;  // points whose quantiles set the grid lines
-constexpr int kZMaxLines = 256;
-static_assert(kCoopThreads == kZSample, "one sample per thread");
-
-// Grid cell of a point: leading bits first, objectives interleaved.
-template <class Coord>
-__device__ __forceinline__ uint32_t z_cell(const float (*s_line)[kZMaxLines], int m, int bits, Coord f)
-{
-    uint32_t c[kTreeMaxM];
-#pragma unroll
-    for (int k = 0; k < kTreeMaxM; ++k) {
-        c[k] = 0u;
-        if (k < m) {
-            const float x = f(k);
-            for (int step = 1 << (bits - 1); step > 0; step >>= 1)
-                if (s_line[k][c[k] + step - 1] <= x) c[k] += step;
-        }
-    }
-    uint32_t key = 0u;
-    for (int b = bits - 1; b >= 0; --b)
-#pragma unroll
-        for (int k = 0; k < kTreeMaxM; ++k)
-            if (k < m) key = key << 1 | ((c[k] >> b) & 1u);
-    return key;
-}
-
-// Points in cell order: lines, counts (an atomic per point, whose old value is
-// the point's slot in its cell), offsets, placement. The order inside a cell
-// depends on the run; ranks do not.
-__global__ void __launch_bounds__(kCoopThreads, 1) k_zorder(Plan* plan)
-{
-    const Group g = group_of(plan, GRP_NARROW);
-    if (g.prob < 0) return;  // a CTA beyond every problem's group
-    const ProbDev& d = plan->p[g.prob];
-    const ProbIn& in = d.in;
-    const long long budget = plan->spin_budget;
-    if (!d.tree || ld_volatile(&d.sc->status) != 0) return;
-    __shared__ float s_smp[2][kZSample];
-    __shared__ float s_line[kTreeMaxM][kZMaxLines];
-    __shared__ int s_warp[33];
-    const int tid = threadIdx.x, m = in.m, bits = d.zbits;
-    const int64_t n2 = in.n2;
-    const float* F = in.F;
-
-    // grid lines: quantiles of a strided sample, two objectives sorted at once
-    const int ns = (int)min((int64_t)kZSample, n2);
-    for (int k0 = 0; k0 < m; k0 += 2) {
-        const int64_t src = (int64_t)tid * n2 / ns;
-        for (int h = 0; h < 2; ++h)
-            s_smp[h][tid] = tid < ns && k0 + h < m ? F[src * m + k0 + h] + 0.0f : INFINITY;
-        __syncthreads();
-        const int t = tid & (kZSample / 2 - 1);
-        float* v = s_smp[tid / (kZSample / 2)];
-        for (int size = 2; size <= kZSample; size <<= 1)
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                const int i = 2 * t - (t & (stride - 1)), j = i + stride;
-                const float a = v[i], b = v[j];
-                if ((a > b) == ((i & size) == 0)) { v[i] = b; v[j] = a; }
-                __syncthreads();
-            }
-        for (int e = tid; e < 2 * kZMaxLines; e += blockDim.x) {
-            const int h = e / kZMaxLines, b = e % kZMaxLines;
-            if (k0 + h < m && b < (1 << bits) - 1) s_line[k0 + h][b] = s_smp[h][(int64_t)(b + 1) * ns >> bits];
-        }
-        __syncthreads();
-    }
-
-    const int64_t t0 = (int64_t)g.rank * blockDim.x + tid, stride = (int64_t)g.size * blockDim.x;
-    for (int64_t i = t0; i < n2; i += stride) {
-        const uint32_t key = z_cell(s_line, m, bits, [&](int k) { return F[i * m + k] + 0.0f; });
-        d.zcell[i] = key;
-        d.zslot[i] = atomicAdd(&d.zcnt[key], 1u);
-    }
-    if (!group_sync(g, d.sc, budget)) return;
-
-    // offsets: exclusive scan of the cell counts over the group
-    {
-        constexpr int PER = 4;
-        const int64_t nc = d.ncell, tile = (int64_t)PER * blockDim.x;
-        const int64_t chunk = cdiv(cdiv(nc, g.size), PER) * PER;
-        const int64_t lo = min(nc, chunk * g.rank), hi = min(nc, lo + chunk);
-        int sum = 0;
-        for (int64_t c = lo + tid; c < hi; c += blockDim.x) sum += (int)__ldcg(&d.zcnt[c]);
-        sum = block_reduce_sum<kCoopThreads>(sum, s_warp);
-        if (tid == 0) d.hist[g.rank] = sum;
-        if (!group_sync(g, d.sc, budget)) return;
-        int base = 0;
-        for (int c = tid; c < g.rank; c += blockDim.x) base += __ldcg(&d.hist[c]);
-        base = block_reduce_sum<kCoopThreads>(base, s_warp);
-        for (int64_t c0 = lo; c0 < hi; c0 += tile) {
-            int v[PER], s = 0;
-#pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                const int64_t c = c0 + (int64_t)tid * PER + e;
-                v[e] = c < hi ? (int)__ldcg(&d.zcnt[c]) : 0;
-                s += v[e];
-            }
-            int tot, run = base + block_exclusive_scan<kCoopThreads>(s, s_warp, tot);
-#pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                const int64_t c = c0 + (int64_t)tid * PER + e;
-                if (c < hi) d.zcnt[c] = (uint32_t)run;
-                run += v[e];
-            }
-            base += tot;
-        }
-        if (!group_sync(g, d.sc, budget)) return;
-    }
-
-    const int64_t zs = (int64_t)d.nleaf * 32;
-    for (int64_t i = t0; i < n2; i += stride) {
-        const uint32_t key = d.zcell[i];  // this thread's own
-        const int64_t pos = (int64_t)__ldcg(&d.zcnt[key]) + d.zslot[i];
-        for (int k = 0; k < m; ++k) d.zpts[k * zs + pos] = F[i * m + k] + 0.0f;
-        d.zidx[pos] = (int32_t)i;
-        d.zkey[pos] = key;
-    }
-}
 
 // ------------------------------------------------------------ k_fronts
 constexpr int kFrontRound = 128;       // leaves of a CTA looked at before their searches run

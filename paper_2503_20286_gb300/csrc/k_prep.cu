@@ -142,6 +142,7 @@ __global__ void k_prep(Plan* plan)
         d.flag[s] = 0;
     }
     for (int64_t c = tid; c < d.ncell; c += stride) d.zcnt[c] = 0u;
+    for (int64_t c = tid; c < 2 * (int64_t)d.nrcell; c += stride) d.rcnt[c] = 0u;
     for (int64_t i = tid; i < n2; i += stride) d.rank_o[i] = kNotRanked;
     if (!d.tree) {
         for (int64_t c = tid; c < 3 * (int64_t)d.ncb; c += stride) d.front_n[c] = 0;
@@ -170,37 +171,9 @@ __global__ void k_prep(Plan* plan)
             for (int k = 0; k < m; ++k) d.rhat[j * m + k] = (float)((double)in.R[j * m + k] * inv);
             d.rho[j] = 0;
             d.lcnt[j] = 0;
-            d.rord[j] = (int32_t)j;
         }
     }
     if (bad) set_status(d.sc, EMO_ERR_NONFINITE);
-}
-
-// References in order of their polar angle from axis 1 (the index of the
-// association scan), their angles from axes 1 and 2 and unit directions in
-// that order.
-__device__ void sort_references(const ProbDev& d, const Group& g, long long budget, RadixSmem& rsm)
-{
-    const int nr = d.in.n_r, m = d.in.m;
-    const int gr = (int)max((int64_t)1, min((int64_t)g.size, cdiv(nr, 4096)));
-    const float* rhat = d.rhat;
-    auto rkey = [&](int32_t j) { return float_key(polar_angle(rhat + (int64_t)j * m, m)); };
-    int rb = 0;
-    for (int shift = 0; shift < 32; shift += kRadixBits) {
-        bool skipped = false;
-        if (!radix_pass(d, g, gr, budget, nr, d.rord + (int64_t)rb * nr, d.rord + (int64_t)(rb ^ 1) * nr, shift, rkey,
-                        skipped, rsm))
-            return;
-        if (!skipped) rb ^= 1;
-    }
-    if (g.rank == 0 && threadIdx.x == 0) d.sc->rbuf = rb;
-    const int32_t* ro = d.rord + (int64_t)rb * nr;
-    for (int64_t s = (int64_t)g.rank * blockDim.x + threadIdx.x; s < nr; s += (int64_t)g.size * blockDim.x) {
-        const int64_t j = __ldcg(&ro[s]);
-        d.rphi[s] = polar_angle(rhat + j * m, m);
-        d.rphi2[s] = polar_angle2(rhat + j * m, m);
-        for (int k = 0; k < m; ++k) d.rsort[s * m + k] = rhat[j * m + k];
-    }
 }
 
 // Lexicographic order, sorted objective keys and runs of equal points.
@@ -217,10 +190,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
     const int gs = (int)max((int64_t)1, min((int64_t)g.size, cdiv(n2, 4096)));
     const float* F = in.F;
     __shared__ RadixSmem rsm;
-    if (!lex_ordered(in)) {  // ranks given, or ranked by the z-order tree: no lexicographic order of the points
-        if (in.mode == MODE_SELECT) sort_references(d, g, budget, rsm);
-        return;
-    }
+    if (!lex_ordered(in)) return;  // ranks given, or ranked by the z-order tree
 
     // Lexicographic order of (f_1, ..., f_m), ties by index. First a stable
     // radix sort by f_1; then every run of equal f_1 (almost always short for
@@ -361,12 +331,6 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
         carry = tmax;
         __syncthreads();
     }
-
-    // every CTA has read the run-start carries from d.hist before the radix
-    // passes of the references reuse it
-    if (in.mode != MODE_SELECT) return;
-    if (!group_sync(g, d.sc, budget)) return;
-    sort_references(d, g, budget, rsm);
 }
 
 }  // namespace emo

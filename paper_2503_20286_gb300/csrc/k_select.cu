@@ -10,13 +10,13 @@
 //     FP32 error band are re-evaluated in FP64;
 //   * hyperplane intercepts: Gaussian elimination with partial pivoting in
 //     FP64 on one thread (m <= 16), nadir fallback;
-//   * association: an FP32 scan over all references keeps the three largest
-//     projections f.r/|r|; references whose projection lies within a
-//     rigorous error band of the best are re-evaluated with the FP64
-//     perpendicular distance d^2 = sum (f_k - t r_k)^2, t = f.r / r.r.
+//   * association: an FP32 search keeps the three smallest distances; references
+//     whose distance lies within a rigorous error band of the best are
+//     re-evaluated with the FP64 perpendicular distance d^2 = sum (f_k - t r_k)^2,
+//     t = f.r / r.r.
 #include "emo_kernels.cuh"
 #include "emo_launch.cuh"
-#include "group_radix.cuh"
+#include "cell_order.cuh"
 
 namespace emo {
 
@@ -45,232 +45,296 @@ __device__ __forceinline__ unsigned long long dbits(double x) { return (unsigned
 
 // ------------------------------------------------------------ k_stats
 // Ideal point, ASF extreme points, nadir point, intercepts (Algorithm S.5).
-__global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
+// Minima and maxima are kept per thread, reduced per warp, then per CTA; the
+// FP64 elimination runs on one warp, a lane per row, every element by the
+// operations of the plain loops in their order.
+struct StatsSmem {
+    uint32_t u[2][kMaxM];
+    unsigned long long best[kMaxM];
+    float z[kMaxM], lim[kMaxM];
+    double A[kMaxM][kMaxM + 1], b[kMaxM];  // column m: right-hand side
+    int warp[33];
+};
+
+// FP32 achievement scalarising function of axis j: max of dev_j and
+// 1e6 dev_k, k != j (top: the largest 1e6 dev_k, at `arg`; second: the next).
+struct AsfTop {
+    float top = 0.0f, second = 0.0f;
+    int arg = -1;
+    __device__ __forceinline__ void add(float a, int k)
+    {
+        if (a > top) {
+            second = top;
+            top = a;
+            arg = k;
+        } else {
+            second = fmaxf(second, a);
+        }
+    }
+    __device__ __forceinline__ float asf(float dev, int j) const { return fmaxf(dev, j == arg ? second : top); }
+};
+
+// MM: objectives at compile time, or kMaxM for any m.
+template <int MM>
+__device__ __noinline__ bool stats_body(const ProbDev& d, const Group& g, long long budget, StatsSmem& sm)
 {
-    const Group g = group_of(plan, GRP_NARROW);
-    if (g.prob < 0) return;  // a CTA beyond every problem's group
-    const ProbDev& d = plan->p[g.prob];
     const ProbIn& in = d.in;
-    const long long budget = plan->spin_budget;
-    if (in.mode != MODE_SELECT || ld_volatile(&d.sc->status) != 0) return;
     Scal* sc = d.sc;
-    const int m = in.m, tid = threadIdx.x, lane = tid & 31;
+    const int m = MM == kMaxM ? in.m : MM, tid = threadIdx.x, lane = tid & 31;
     const int nS = ld_volatile(&sc->nS);
     const float* F = in.F;
     const int64_t stride = (int64_t)g.size * blockDim.x;
     const int64_t t0 = (int64_t)g.rank * blockDim.x + tid;
-    __shared__ uint32_t s_u32[kMaxM];
-    __shared__ unsigned long long s_u64[kMaxM];
-    __shared__ float s_z[kMaxM];
 
-    // 1. ideal point: keep ~key maxima (Scal is zero-initialised)
-    if (tid < kMaxM) s_u32[tid] = 0u;
+    // 1. ideal point and largest objectives (~key and key maxima; Scal is zero-initialised)
+    if (tid < kMaxM) sm.u[0][tid] = sm.u[1][tid] = 0u;
     __syncthreads();
     {
-        uint32_t best[kMaxM];
+        uint32_t lo[MM], hi[MM];
 #pragma unroll
-        for (int k = 0; k < kMaxM; ++k) best[k] = 0u;
+        for (int k = 0; k < MM; ++k) lo[k] = hi[k] = 0u;
         for (int64_t i = t0; i < nS; i += stride) {
             const int64_t v = d.slist[i];
 #pragma unroll
-            for (int k = 0; k < kMaxM; ++k)
-                if (k < m) best[k] = max(best[k], ~float_key(F[v * m + k]));
+            for (int k = 0; k < MM; ++k)
+                if (k < m) {
+                    const uint32_t key = float_key(F[v * m + k]);
+                    lo[k] = max(lo[k], ~key);
+                    hi[k] = max(hi[k], key);
+                }
         }
 #pragma unroll
-        for (int k = 0; k < kMaxM; ++k) {
-            if (k >= m) break;
-            uint32_t b = best[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-            if (lane == 0 && b) atomicMax(&s_u32[k], b);
-        }
+        for (int k = 0; k < MM; ++k)
+            if (k < m) {
+                const uint32_t a = __reduce_max_sync(0xffffffffu, lo[k]), b = __reduce_max_sync(0xffffffffu, hi[k]);
+                if (lane == 0 && b) {
+                    atomicMax(&sm.u[0][k], a);
+                    atomicMax(&sm.u[1][k], b);
+                }
+            }
     }
     __syncthreads();
-    if (tid < m && s_u32[tid]) atomicMax(&sc->zkey[tid], s_u32[tid]);
-    if (!group_sync(g, sc, budget)) return;
-    if (tid < m) s_z[tid] = key_float(~__ldcg(&sc->zkey[tid]));
-    if (tid < kMaxM) { s_u32[tid] = 0u; s_u64[tid] = 0ull; }
+    if (tid < m && sm.u[1][tid]) {
+        atomicMax(&sc->zkey[tid], sm.u[0][tid]);
+        atomicMax(&sc->fkey[tid], sm.u[1][tid]);
+    }
+    if (!group_sync(g, sc, budget)) return false;
+    if (tid < m) sm.z[tid] = key_float(~__ldcg(&sc->zkey[tid]));
+    if (tid < kMaxM) sm.u[0][tid] = 0u;
     __syncthreads();
+    float z[MM];
+#pragma unroll
+    for (int k = 0; k < MM; ++k) z[k] = k < m ? sm.z[k] : 0.0f;
+    auto devs = [&](int64_t v, float (&dev)[MM]) {
+        AsfTop t;
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+            dev[k] = k < m ? F[v * m + k] - z[k] : 0.0f;
+            if (k < m) t.add(dev[k] * 1.0e6f, k);
+        }
+        return t;
+    };
 
-    // 2. FP32 ASF minima per axis (stored as ~bits maxima) and FP64 nadir
+    // 2. FP32 ASF minima per axis (stored as ~bits maxima)
     {
+        float best[MM];
+#pragma unroll
+        for (int k = 0; k < MM; ++k) best[k] = INFINITY;
         for (int64_t i = t0; i < nS; i += stride) {
-            const int64_t v = d.slist[i];
-            float dev[kMaxM];
+            float dev[MM];
+            const AsfTop t = devs(d.slist[i], dev);
 #pragma unroll
-            for (int k = 0; k < kMaxM; ++k) dev[k] = k < m ? F[v * m + k] - s_z[k] : 0.0f;
-#pragma unroll
-            for (int k = 0; k < kMaxM; ++k) {
-                if (k >= m) break;
-                const double nd = __dsub_rn((double)F[v * m + k], (double)s_z[k]);
-                atomicMax(&s_u64[k], dbits(nd));
-            }
-            for (int j = 0; j < m; ++j) {
-                float asf = 0.0f;
-#pragma unroll
-                for (int k = 0; k < kMaxM; ++k)
-                    if (k < m) asf = fmaxf(asf, k == j ? dev[k] : dev[k] * 1.0e6f);
-                atomicMax(&s_u32[j], ~__float_as_uint(asf));
-            }
+            for (int k = 0; k < MM; ++k) best[k] = fminf(best[k], t.asf(dev[k], k));
         }
+#pragma unroll
+        for (int k = 0; k < MM; ++k)
+            if (k < m) {
+                const uint32_t b = __reduce_max_sync(0xffffffffu, ~__float_as_uint(best[k]));
+                if (lane == 0) atomicMax(&sm.u[0][k], b);
+            }
     }
     __syncthreads();
-    if (tid < m) {
-        atomicMax(&sc->asf32[tid], s_u32[tid]);
-        atomicMax(&sc->nadir[tid], s_u64[tid]);
-    }
-    if (!group_sync(g, sc, budget)) return;
+    if (tid < m) atomicMax(&sc->asf32[tid], sm.u[0][tid]);
+    if (!group_sync(g, sc, budget)) return false;
 
     // 3. exact FP64 ASF of the candidates within the FP32 error band
-    if (tid < kMaxM) s_u64[tid] = 0ull;
-    __syncthreads();
-    __shared__ float s_lim[kMaxM];
+    if (tid < kMaxM) sm.best[tid] = 0ull;
     if (tid < m) {
         const float mn = __uint_as_float(~__ldcg(&sc->asf32[tid]));
-        s_lim[tid] = mn * (1.0f + 0x1p-18f) + 1e-30f;
+        sm.lim[tid] = mn * (1.0f + 0x1p-18f) + 1e-30f;
     }
     __syncthreads();
     auto asf64 = [&](int64_t v, int j) {
         double mx = -INFINITY;
         for (int k = 0; k < m; ++k) {
             const double w = k == j ? 1.0 : 1e-6;
-            const double t = __ddiv_rn(__dsub_rn((double)F[v * m + k], (double)s_z[k]), w);
+            const double t = __ddiv_rn(__dsub_rn((double)F[v * m + k], (double)sm.z[k]), w);
             if (t > mx) mx = t;
         }
         return mx;
     };
-    auto asf32 = [&](int64_t v, int j) {
-        float asf = 0.0f;
-        for (int k = 0; k < m; ++k) {
-            const float dv = F[v * m + k] - s_z[k];
-            asf = fmaxf(asf, k == j ? dv : dv * 1.0e6f);
-        }
-        return asf;
-    };
     for (int64_t i = t0; i < nS; i += stride) {
         const int64_t v = d.slist[i];
-        for (int j = 0; j < m; ++j)
-            if (asf32(v, j) <= s_lim[j]) atomicMax(&s_u64[j], ~dbits(asf64(v, j)));
+        float dev[MM];
+        const AsfTop t = devs(v, dev);
+#pragma unroll
+        for (int k = 0; k < MM; ++k)
+            if (k < m && t.asf(dev[k], k) <= sm.lim[k]) atomicMax(&sm.best[k], ~dbits(asf64(v, k)));
     }
     __syncthreads();
-    if (tid < m) atomicMax(&sc->asf64[tid], s_u64[tid]);
-    if (!group_sync(g, sc, budget)) return;
+    if (tid < m && sm.best[tid]) atomicMax(&sc->asf64[tid], sm.best[tid]);
+    if (!group_sync(g, sc, budget)) return false;
 
     // 4. lowest index attaining the FP64 minimum (stored as INT32_MAX - i maxima)
-    __shared__ unsigned long long s_best[kMaxM];
-    if (tid < m) s_best[tid] = ~__ldcg(&sc->asf64[tid]);
+    if (tid < m) sm.best[tid] = ~__ldcg(&sc->asf64[tid]);
     __syncthreads();
     for (int64_t i = t0; i < nS; i += stride) {
         const int64_t v = d.slist[i];
-        for (int j = 0; j < m; ++j)
-            if (asf32(v, j) <= s_lim[j] && dbits(asf64(v, j)) == s_best[j])
-                atomicMax(&sc->ext[j], INT32_MAX - (int)v);
+        float dev[MM];
+        const AsfTop t = devs(v, dev);
+#pragma unroll
+        for (int k = 0; k < MM; ++k)
+            if (k < m && t.asf(dev[k], k) <= sm.lim[k] && dbits(asf64(v, k)) == sm.best[k])
+                atomicMax(&sc->ext[k], INT32_MAX - (int)v);
     }
-    if (!group_sync(g, sc, budget)) return;
+    if (!group_sync(g, sc, budget)) return false;
 
     // 5. intercepts by Gaussian elimination with partial pivoting (FP64)
-    if (g.rank == 0 && tid == 0) {
-        double A[kMaxM][kMaxM], rhs[kMaxM], b[kMaxM], a[kMaxM];
-        int ext[kMaxM];
-        double maxabs = 0.0;
-        for (int j = 0; j < m; ++j) {
-            const int e = ld_volatile(&sc->ext[j]);
-            if (e <= 0) {  // no candidate attained the minimum (non-finite values)
-                set_status(sc, EMO_ERR_NONFINITE);
-                return;
+    if (g.rank == 0 && tid < 32) {
+        const int e = lane < m ? ld_volatile(&sc->ext[lane]) : 1;
+        if (__any_sync(0xffffffffu, e <= 0)) {  // no candidate attained the minimum (non-finite values)
+            if (lane == 0) set_status(sc, EMO_ERR_NONFINITE);
+        } else {
+            const int ext = INT32_MAX - e;
+            double maxabs = 0.0;
+            if (lane < m) {
+                for (int k = 0; k < m; ++k) {
+                    const double x = __dsub_rn((double)F[(int64_t)ext * m + k], (double)sm.z[k]);
+                    sm.A[lane][k] = x;
+                    maxabs = fmax(maxabs, fabs(x));
+                }
+                sm.A[lane][m] = 1.0;
             }
-            ext[j] = INT32_MAX - e;
-            rhs[j] = 1.0;
-            for (int k = 0; k < m; ++k) {
-                A[j][k] = __dsub_rn((double)F[(int64_t)ext[j] * m + k], (double)s_z[k]);
-                maxabs = fmax(maxabs, fabs(A[j][k]));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) maxabs = fmax(maxabs, __shfl_xor_sync(0xffffffffu, maxabs, o));
+            __syncwarp();
+            bool singular = false;
+            for (int col = 0; col < m; ++col) {
+                int piv = col;
+                for (int r = col + 1; r < m; ++r)
+                    if (fabs(sm.A[r][col]) > fabs(sm.A[piv][col])) piv = r;
+                if (!(fabs(sm.A[piv][col]) > __dmul_rn(1e-12, maxabs))) {
+                    singular = true;
+                    break;
+                }
+                __syncwarp();
+                if (piv != col && lane <= m) {
+                    const double t = sm.A[col][lane];
+                    sm.A[col][lane] = sm.A[piv][lane];
+                    sm.A[piv][lane] = t;
+                }
+                __syncwarp();
+                if (lane > col && lane < m) {
+                    const double f = __ddiv_rn(sm.A[lane][col], sm.A[col][col]);
+                    for (int c = col; c <= m; ++c)
+                        sm.A[lane][c] = __dsub_rn(sm.A[lane][c], __dmul_rn(f, sm.A[col][c]));
+                }
+                __syncwarp();
             }
+            double a = 1.0;
+            bool fallback = singular;
+            if (!singular) {
+                for (int col = m - 1; col >= 0; --col) {
+                    double s = sm.A[col][m];
+                    for (int c = col + 1; c < m; ++c) s = __dsub_rn(s, __dmul_rn(sm.A[col][c], sm.b[c]));
+                    s = __ddiv_rn(s, sm.A[col][col]);
+                    __syncwarp();
+                    if (lane == 0) sm.b[col] = s;
+                    __syncwarp();
+                }
+                if (lane < m) a = __ddiv_rn(1.0, sm.b[lane]);
+                fallback = __any_sync(0xffffffffu, lane < m && (!isfinite(a) || a <= 1e-10));
+            }
+            if (lane < m) {
+                if (fallback) {  // the nadir point: the largest F_k - z_k of S
+                    a = __dsub_rn((double)key_float(__ldcg(&sc->fkey[lane])), (double)sm.z[lane]);
+                    if (a <= 1e-10) a = 1.0;
+                }
+                sc->a[lane] = a;
+                sc->inv_a32[lane] = (float)__ddiv_rn(1.0, a);
+                sc->z[lane] = sm.z[lane];
+                sc->ext[lane] = ext;
+            }
+            if (lane == 0) sc->fallback = fallback;
         }
-        int singular = 0;
-        for (int col = 0; col < m && !singular; ++col) {
-            int piv = col;
-            for (int r = col + 1; r < m; ++r)
-                if (fabs(A[r][col]) > fabs(A[piv][col])) piv = r;
-            if (!(fabs(A[piv][col]) > __dmul_rn(1e-12, maxabs))) { singular = 1; break; }
-            if (piv != col) {
-                for (int c = 0; c < m; ++c) { double t = A[col][c]; A[col][c] = A[piv][c]; A[piv][c] = t; }
-                double t = rhs[col]; rhs[col] = rhs[piv]; rhs[piv] = t;
-            }
-            for (int r = col + 1; r < m; ++r) {
-                const double f = __ddiv_rn(A[r][col], A[col][col]);
-                for (int c = col; c < m; ++c) A[r][c] = __dsub_rn(A[r][c], __dmul_rn(f, A[col][c]));
-                rhs[r] = __dsub_rn(rhs[r], __dmul_rn(f, rhs[col]));
-            }
-        }
-        int fallback = singular;
-        if (!singular) {
-            for (int col = m - 1; col >= 0; --col) {
-                double s = rhs[col];
-                for (int c = col + 1; c < m; ++c) s = __dsub_rn(s, __dmul_rn(A[col][c], b[c]));
-                b[col] = __ddiv_rn(s, A[col][col]);
-            }
-            for (int k = 0; k < m; ++k) {
-                a[k] = __ddiv_rn(1.0, b[k]);
-                if (!isfinite(a[k]) || a[k] <= 1e-10) fallback = 1;
-            }
-        }
-        if (fallback) {
-            for (int k = 0; k < m; ++k) {
-                a[k] = __longlong_as_double((long long)__ldcg(&sc->nadir[k]));
-                if (a[k] <= 1e-10) a[k] = 1.0;
-            }
-        }
-        for (int k = 0; k < m; ++k) {
-            sc->a[k] = a[k];
-            sc->inv_a32[k] = (float)__ddiv_rn(1.0, a[k]);
-            sc->z[k] = s_z[k];
-            sc->ext[k] = ext[k];
-        }
-        sc->fallback = fallback;
-        __threadfence();
     }
 
-    // 6. S in the order of the polar angle of its normalised points (16-bit
-    // buckets, two radix passes): neighbouring threads of the association
-    // then scan neighbouring references. Any order of S gives the same result.
-    if (!group_sync(g, sc, budget)) return;
-    __shared__ RadixSmem rsm;
-    float zf[kMaxM], ia[kMaxM];
-    for (int k = 0; k < m; ++k) {
-        zf[k] = __ldcg(&sc->z[k]);
-        ia[k] = __ldcg(&sc->inv_a32[k]);
+    // 6. S in the order of the references' grid cells (direction of the
+    // normalised point), so that the points of an association warp look at the
+    // same references. Any order of S gives the same result.
+    if (!group_sync(g, sc, budget)) return false;
+    __shared__ DirGrid s_grid;
+    if (tid < kMaxM) {
+        s_grid.lo[tid] = d.rgrid->lo[tid];
+        s_grid.scale[tid] = d.rgrid->scale[tid];
     }
-    auto akey = [&](int32_t v) {
-        float f[kMaxM];
-        for (int k = 0; k < m; ++k) f[k] = (F[(int64_t)v * m + k] - zf[k]) * ia[k];
-        const int b = (int)(polar_angle(f, m) * (65535.0f / 1.5707964f));
-        return (uint32_t)(b < 0 ? 0 : (b > 65535 ? 65535 : b));
-    };
-    int32_t* bufs[2] = {d.slist, d.llist};
-    int cur = 0;
-    const int gsS = (int)max((int64_t)1, min((int64_t)g.size, cdiv(nS, 4096)));
-    for (int shift = 0; shift < 16; shift += kRadixBits) {
-        bool skipped = false;
-        if (!radix_pass(d, g, gsS, budget, nS, bufs[cur], bufs[cur ^ 1], shift, akey, skipped, rsm)) return;
-        if (!skipped) cur ^= 1;
-    }
-    if (cur == 1) {
-        for (int64_t i = t0; i < nS; i += stride) d.slist[i] = __ldcg(&d.llist[i]);
-        group_sync(g, sc, budget);
+    float ia[MM];
+#pragma unroll
+    for (int k = 0; k < MM; ++k) ia[k] = k < m ? __ldcg(&sc->inv_a32[k]) : 0.0f;
+    __syncthreads();
+    const CellSort cs{nS, d.nrcell, d.rcnt + d.nrcell, d.scell, d.sslot};
+    cell_count(cs, g, [&](int64_t i) {
+        const int64_t v = d.slist[i];
+        float f[MM], n2 = 0.0f;
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+            f[k] = k < m ? (F[v * m + k] - z[k]) * ia[k] : 0.0f;
+            n2 = fmaf(f[k], f[k], n2);
+        }
+        const float inv = rsqrtf(n2);
+        return dir_cell(s_grid, m, d.rbits, [&](int k) { return f[k] * inv; });
+    });
+    if (!group_sync(g, sc, budget)) return false;
+    cell_total(cs, g, d.hist, sm.warp);
+    if (!group_sync(g, sc, budget)) return false;
+    cell_offsets(cs, g, d.hist, sm.warp);
+    if (!group_sync(g, sc, budget)) return false;
+    cell_place(cs, g, [&](int64_t i, uint32_t, int64_t pos) { d.sord[pos] = d.slist[i]; });
+    return true;
+}
+
+__global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
+{
+    __shared__ StatsSmem sm;
+    const Group g = group_of(plan, GRP_NARROW);
+    if (g.prob < 0) return;  // a CTA beyond every problem's group
+    const ProbDev& d = plan->p[g.prob];
+    if (d.in.mode != MODE_SELECT || ld_volatile(&d.sc->status) != 0) return;
+    switch (d.in.m) {
+    case 2: stats_body<2>(d, g, plan->spin_budget, sm); break;
+    case 3: stats_body<3>(d, g, plan->spin_budget, sm); break;
+    case 4: stats_body<4>(d, g, plan->spin_budget, sm); break;
+    case 5: stats_body<5>(d, g, plan->spin_budget, sm); break;
+    default: stats_body<kMaxM>(d, g, plan->spin_budget, sm);
     }
 }
 
 // ------------------------------------------------------------ association
 // FP32 scan: the perpendicular distance is computed in the cancellation-free
 // form d^2 = sum_k (f_k - g u_k)^2, g = f.u, u = r/|r| (linear in the angle
-// near the optimum, so its error band is narrow). Candidates come from the
-// angular index: references sorted by polar angle phi from axis 1; since the
-// angle between two directions is at least the difference of their polar
-// angles (triangle inequality on the sphere), only references with
-// |phi_r - phi_f| <= theta_best + margin can beat the best one found so far.
-// The scan walks outward from phi_f and stops on that bound. The same
-// inequality for the angle from axis 2 (a second pivot, stored per reference)
-// skips the distance of references on the far side of the band's ring.
+// near the optimum, so its error band is narrow). References are visited
+// through the two-level tree of balls that k_order built over the unit
+// directions: a warp takes neighbouring points of S (any objective count; the
+// fewer points there are, the more lanes share one), finds the leaf nearest to
+// their mean direction, then every leaf whose ball may hold a reference nearer
+// than the best so far to one of them: |p - c| <= R + b, with p the point's
+// unit direction, c and R the ball and b the chord of the best angle (plus a
+// margin). A leaf's 32 references pass through shared memory.
+// Bound by issue and the latency of the leaves' tests. Measured (association
+// and decision together): 200,864 points on 200,028 references, m = 3, 0.33 ms
+// (0.43 ms by a scan outward from each point's polar angle); 22,170 points on
+// 20,475 references, m = 5, 0.26 ms (0.79 ms visiting every reference); 10,056
+// on 10,011, m = 3, 53 us (92 us).
 //
 // Error band of the FP32 distance (relative to |f|), two evaluations:
 // |delta d| <= (sqrt(m)(m + 10) + (m + 1)/2) u |f| each.
@@ -278,10 +342,10 @@ __device__ __forceinline__ float assoc_band(int m)
 {
     return (2.0f * sqrtf((float)m) * (float)(m + 10) + (float)(m + 8)) * 1.05f * 0x1p-24f;
 }
-// Extra angular margin of the index scan: covers the atan2/asin rounding and
-// keeps every unscanned reference farther than the band from the best.
+// Extra margin of the search: covers the rounding of the directions, balls
+// and chords and keeps every unvisited reference farther than the band from
+// the best.
 __device__ __forceinline__ float assoc_margin(int m) { return 1e-5f + 8.0f * assoc_band(m); }
-constexpr float kAssocMaxBound = 0.7853981f;  // beyond pi/4 the scan covers every reference
 
 template <int M>
 __device__ __forceinline__ float d2_f32(const float* f, const float* u)
@@ -298,392 +362,310 @@ __device__ __forceinline__ float d2_f32(const float* f, const float* u)
     return d2;
 }
 
-// Exact decision between candidate references (FP64, reference formula).
-__device__ inline void decide64(const ProbDev& d, const Scal* sc, int64_t v, int m, const int* cand, int nc,
-                                int& best_j, double& best_d2)
-{
-    double fn[kMaxM];
-    for (int k = 0; k < m; ++k) fn[k] = fnorm64(d.in.F[v * m + k], sc->z[k], sc->a[k]);
-    best_j = -1;
-    best_d2 = INFINITY;
-    for (int c = 0; c < nc; ++c) {
-        const int j = cand[c];
-        const double d2 = perp_d2(fn, d.in.R + (int64_t)j * m, m);
-        if (d2 < best_d2 || (d2 == best_d2 && j < best_j)) { best_d2 = d2; best_j = j; }
-    }
-}
-
-// First sorted position with rphi >= x.
-__device__ __forceinline__ int lower_bound_f(const float* a, int n, float x)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(&a[mid]) < x) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-template <int M>
-__global__ void __launch_bounds__(256) k_assoc_m(Plan* plan, int pfirst, int plast)
-{
-    // the points of S of every problem of this m in one sequence (a batch's
-    // small problems together fill the grid)
-    __shared__ long long s_first[kMaxBatch + 1];
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        long long acc = 0;
-        for (int p = pfirst; p < plast; ++p) {
-            s_first[p - pfirst] = acc;
-            const ProbDev& d = plan->p[p];
-            if (d.in.mode == MODE_SELECT && d.in.m == M && ld_volatile(&d.sc->status) == 0)
-                acc += ld_volatile(&d.sc->nS);
-        }
-        s_first[plast - pfirst] = acc;
-    }
-    __syncthreads();
-    const long long total = s_first[plast - pfirst];
-    const float band = assoc_band(M), margin = assoc_margin(M);
-    // a population split over GPUs associates only its own points
-    const bool ranged = plan->split.kind == SPLIT_ASSOC;
-    for (long long gs = (long long)blockIdx.x * 256 + tid; gs < total; gs += (long long)gridDim.x * 256) {
-        int plo = 0, phi = plast - pfirst;  // last problem with s_first <= gs
-        while (phi - plo > 1) {
-            const int mid = (plo + phi) >> 1;
-            if (s_first[mid] <= gs) plo = mid;
-            else phi = mid;
-        }
-        while (s_first[plo + 1] <= gs) ++plo;  // skip problems without points
-        const ProbDev& d = plan->p[pfirst + plo];
-        const Scal* sc = d.sc;
-        const int64_t s = gs - s_first[plo];
-        const int nr = d.in.n_r;
-        const float* __restrict__ rphi = d.rphi;
-        const float* __restrict__ rphi2 = d.rphi2;
-        const float* __restrict__ rs = d.rsort;
-        const int32_t* __restrict__ ro = d.rord + (int64_t)sc->rbuf * nr;
-        const int64_t lo = ranged ? plan->split.col_lo : 0, hi = ranged ? plan->split.col_hi : d.in.n2;
-        const int64_t v = d.slist[s];
-        if (v < lo || v >= hi) continue;
-        float f[M];
-        float n2 = 0.0f;
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-            f[k] = (d.in.F[v * M + k] - sc->z[k]) * sc->inv_a32[k];
-            n2 = fmaf(f[k], f[k], n2);
-        }
-        const float nrm = sqrtf(n2);
-        if (!(nrm > 0.0f) || !isfinite(nrm)) {  // at the ideal point (or overflow): exhaustive FP64 scan
-            const int slot = atomicAdd(&d.sc->nflag, 1);
-            d.flagged[slot] = (int32_t)v;
-            d.flagged_bound[slot] = INFINITY;
-            continue;
-        }
-        const float phif = polar_angle(f, M);
-        const float phi2f = polar_angle2(f, M);
-        float c1 = INFINITY, c2 = INFINITY, c3 = INFINITY;  // FP32 d^2, best three
-        int s1 = -1, s2 = -1;                                 // sorted positions of the best two
-        float bound = INFINITY;                               // angular half-width still to scan
-        int L = lower_bound_f(rphi, nr, phif) - 1, Rp = L + 1;
-        float dl = L >= 0 ? phif - __ldg(&rphi[L]) : INFINITY;
-        float dr = Rp < nr ? __ldg(&rphi[Rp]) - phif : INFINITY;
-        while (L >= 0 || Rp < nr) {  // at most n_r steps
-            const bool left = L >= 0 && (Rp >= nr || dl <= dr);
-            const float dm = left ? dl : dr;
-            if (!(dm <= bound)) break;
-            int q;  // 0 <= q < n_r
-            if (left) {
-                q = L--;
-                dl = L >= 0 ? phif - __ldg(&rphi[L]) : INFINITY;
-            } else {
-                q = Rp++;
-                dr = Rp < nr ? __ldg(&rphi[Rp]) - phif : INFINITY;
-            }
-            // second pivot: the angle to the reference is at least the
-            // difference of the angles from axis 2 (same margins as axis 1)
-            if (M > 2 && !(fabsf(__ldg(&rphi2[q]) - phi2f) <= bound)) continue;
-            float u[M];
-#pragma unroll
-            for (int k = 0; k < M; ++k) u[k] = __ldg(&rs[(int64_t)q * M + k]);
-            const float dd = d2_f32<M>(f, u);
-            if (dd < c3) {
-                if (dd < c2) {
-                    c3 = c2;
-                    if (dd < c1) { c2 = c1; s2 = s1; c1 = dd; s1 = q; }
-                    else { c2 = dd; s2 = q; }
-                    // angle of the best so far, bounded from above
-                    const float sn = fminf(1.0f, sqrtf(c1) / nrm * 1.00001f + 2.0f * band);
-                    const float th = asinf(sn);
-                    bound = th + margin > kAssocMaxBound ? INFINITY : th + margin;
-                } else {
-                    c3 = dd;
-                }
-            }
-        }
-        const float d1 = sqrtf(c1), lim = d1 + band * nrm;
-        if (sqrtf(c3) <= lim) {  // three or more references inside the band
-            const int slot = atomicAdd(&d.sc->nflag, 1);
-            d.flagged[slot] = (int32_t)v;
-            d.flagged_bound[slot] = bound;
-            continue;
-        }
-        int cand[2];
-        int nc = 0;
-        cand[nc++] = __ldg(&ro[s1]);
-        if (s2 >= 0 && sqrtf(c2) <= lim) cand[nc++] = __ldg(&ro[s2]);
-        int bj;
-        double bd2;
-        decide64(d, sc, v, M, cand, nc, bj, bd2);
-        d.pi[v] = bj;
-        d.d64[v] = __dsqrt_rn(bd2);
-    }
-}
-
-// All-reference association for m >= 4, where the polar-angle index prunes
-// little: every reference is visited, uniformly across a warp. A CTA takes a
-// tile of 64 points of S (two per lane, the same in every warp) and stages
-// the unit directions in shared memory, 1024 (m <= 8) or 512 at a time; warp
-// w visits the w-th eighth of each staged block for the tile's points,
-// keeping the three smallest FP32 distances and the references of the two
-// smallest; the eight warps' lists are merged and the decision is the one of
-// k_assoc_m (two candidates inside the FP32 band: FP64 decision; three or
-// more: the point is re-scanned in FP64 by k_rescan over every reference).
-// Which reference of an FP32 tie is kept does not matter: tied candidates
-// are inside the band together. Tiles are taken from a counter, problems
-// with the most references first. (A per-point angular filter on the
-// projection f.u before the distance was measured slower: the 64 points of
-// a warp rarely all skip the same reference, and the warp runs the distance
-// whenever one of them does not.)
-constexpr int kBfWarps = 8;
-constexpr int kBfPPL = 2;                    // points per lane
-constexpr int kBfTile = 32 * kBfPPL;         // points per CTA tile
-constexpr int kBfStageBytes = 32768;         // staged unit directions
-
-struct BfTop {
+// The three smallest FP32 squared distances, sorted positions of the two smallest.
+struct Top3 {
     float c1, c2, c3;
     int s1, s2;
     __device__ __forceinline__ void init() { c1 = c2 = c3 = INFINITY; s1 = s2 = -1; }
     __device__ __forceinline__ void add(float dd, int j)
     {
         if (dd < c3) {
-            if (dd < c2) {
-                c3 = c2;
-                if (dd < c1) { c2 = c1; s2 = s1; c1 = dd; s1 = j; }
-                else { c2 = dd; s2 = j; }
-            } else {
-                c3 = dd;
-            }
+            const bool b1 = dd < c1, b2 = dd < c2;
+            c3 = b2 ? c2 : dd;
+            s2 = b1 ? s1 : (b2 ? j : s2);
+            c2 = b1 ? c1 : (b2 ? dd : c2);
+            s1 = b1 ? j : s1;
+            c1 = b1 ? dd : c1;
         }
     }
 };
 
+// Chord up to which references have to be visited, given the best d and |f|
+// (infinite beyond an angle of pi / 4).
 template <int M>
-__global__ void __launch_bounds__(kBfWarps * 32) k_assoc_all(Plan* plan, int pfirst, int plast)
+__device__ __forceinline__ float assoc_chord(float c1, float nrm)
 {
-    constexpr int MP = (M + 3) / 4 * 4;  // padded to whole float4
-    constexpr int kStage = kBfStageBytes / (MP * 4);
-    constexpr int kPerWarp = (kStage + kBfWarps - 1) / kBfWarps;
-    __shared__ float4 s_u[kStage * MP / 4];
-    __shared__ float s_c[3][kBfWarps][kBfTile];
-    __shared__ int s_s[2][kBfWarps][kBfTile];
-    __shared__ int s_ord[kMaxBatch], s_first[kMaxBatch + 1];
-    __shared__ int s_np, s_tile;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) {  // problems of this m, most references first; tile prefix
-        int np = 0;
-        for (int p = pfirst; p < plast; ++p) {
-            const ProbDev& d = plan->p[p];
-            if (d.in.mode != MODE_SELECT || d.in.m != M || ld_volatile(&d.sc->status) != 0) continue;
-            int i = np++;
-            while (i > 0 && plan->p[s_ord[i - 1]].in.n_r < d.in.n_r) { s_ord[i] = s_ord[i - 1]; --i; }
-            s_ord[i] = p;
-        }
-        s_first[0] = 0;
-        for (int i = 0; i < np; ++i)
-            s_first[i + 1] = s_first[i] + (int)cdiv(ld_volatile(&plan->p[s_ord[i]].sc->nS), kBfTile);
-        s_np = np;
-    }
-    __syncthreads();
-    const int np = s_np, ntiles = s_first[np];
-    for (;;) {
-        if (tid == 0) s_tile = (int)atomicAdd(&plan->asc_next[M], 1ull);
-        __syncthreads();
-        const int t = s_tile;
-        __syncthreads();  // every thread has read s_tile
-        if (t >= ntiles) break;
-        int pi_ = 0;
-        while (s_first[pi_ + 1] <= t) ++pi_;
-        const ProbDev& d = plan->p[s_ord[pi_]];
-        const Scal* sc = d.sc;
-        const int nS = ld_volatile(&sc->nS), nr = d.in.n_r;
-        const bool ranged = plan->split.kind == SPLIT_ASSOC;
-        const int64_t lo = ranged ? plan->split.col_lo : 0, hi = ranged ? plan->split.col_hi : d.in.n2;
-        const int64_t s0 = (int64_t)(t - s_first[pi_]) * kBfTile;
-        float f[kBfPPL][M];
-        float nrm[kBfPPL];
-        int64_t v[kBfPPL];
-        bool act[kBfPPL];
-        BfTop top[kBfPPL];
-#pragma unroll
-        for (int i = 0; i < kBfPPL; ++i) {
-            const int64_t s = s0 + i * 32 + lane;
-            v[i] = s < nS ? (int64_t)d.slist[s] : -1;
-            act[i] = v[i] >= lo && v[i] < hi;
-            float n2 = 0.0f;
-#pragma unroll
-            for (int k = 0; k < M; ++k) {
-                f[i][k] = act[i] ? (d.in.F[v[i] * M + k] - sc->z[k]) * sc->inv_a32[k] : 0.0f;
-                n2 = fmaf(f[i][k], f[i][k], n2);
-            }
-            nrm[i] = sqrtf(n2);
-            top[i].init();
-        }
-        bool scan = false;
-#pragma unroll
-        for (int i = 0; i < kBfPPL; ++i) scan |= act[i] && nrm[i] > 0.0f && isfinite(nrm[i]);
-        if (__syncthreads_or(scan)) {
-            for (int r0 = 0; r0 < nr; r0 += kStage) {
-                const int cnt = min(kStage, nr - r0);
-                __syncthreads();  // the previous block has been scanned
-                float* su = (float*)s_u;
-                for (int e = tid; e < cnt * MP; e += kBfWarps * 32) {
-                    const int q = e / MP, k = e - q * MP;
-                    su[e] = k < M ? __ldg(&d.rhat[(int64_t)(r0 + q) * M + k]) : 0.0f;
-                }
-                __syncthreads();
-                const int qa = warp * kPerWarp, qb = min(cnt, qa + kPerWarp);
-                for (int q = qa; q < qb; ++q) {
-                    float u[MP];
-#pragma unroll
-                    for (int k4 = 0; k4 < MP / 4; ++k4) {
-                        const float4 x = s_u[q * (MP / 4) + k4];
-                        u[4 * k4] = x.x;
-                        u[4 * k4 + 1] = x.y;
-                        u[4 * k4 + 2] = x.z;
-                        u[4 * k4 + 3] = x.w;
-                    }
-#pragma unroll
-                    for (int i = 0; i < kBfPPL; ++i) top[i].add(d2_f32<M>(f[i], u), r0 + q);
-                }
-            }
-        }
-        // merge the warps' lists; threads 0 .. 63 decide one point each
-#pragma unroll
-        for (int i = 0; i < kBfPPL; ++i) {
-            const int pt = i * 32 + lane;
-            s_c[0][warp][pt] = top[i].c1;
-            s_c[1][warp][pt] = top[i].c2;
-            s_c[2][warp][pt] = top[i].c3;
-            s_s[0][warp][pt] = top[i].s1;
-            s_s[1][warp][pt] = top[i].s2;
-        }
-        __syncthreads();
-        if (tid < kBfTile) {
-            const int64_t s = s0 + tid;  // point tid of the tile (lane tid & 31, slot tid >> 5)
-            const int64_t vv = s < nS ? (int64_t)d.slist[s] : -1;
-            if (vv >= lo && vv < hi) {
-                BfTop b;
-                b.init();
-                for (int w = 0; w < kBfWarps; ++w) {
-                    // the smaller two carry references; a third value only its distance
-                    b.add(s_c[0][w][tid], s_s[0][w][tid]);
-                    b.add(s_c[1][w][tid], s_s[1][w][tid]);
-                    b.add(s_c[2][w][tid], -1);
-                }
-                float ff[M], n2 = 0.0f;
-#pragma unroll
-                for (int k = 0; k < M; ++k) {
-                    ff[k] = (d.in.F[vv * M + k] - sc->z[k]) * sc->inv_a32[k];
-                    n2 = fmaf(ff[k], ff[k], n2);
-                }
-                const float nm = sqrtf(n2);
-                const float band = assoc_band(M);
-                if (!(nm > 0.0f) || !isfinite(nm) || sqrtf(b.c3) <= sqrtf(b.c1) + band * nm) {
-                    // at the ideal point, or three or more references inside the band
-                    const int slot = atomicAdd(&d.sc->nflag, 1);
-                    d.flagged[slot] = (int32_t)vv;
-                    d.flagged_bound[slot] = INFINITY;
-                } else {
-                    const float lim = sqrtf(b.c1) + band * nm;
-                    int cand[2];
-                    int nc = 0;
-                    cand[nc++] = b.s1;
-                    if (b.s2 >= 0 && sqrtf(b.c2) <= lim) cand[nc++] = b.s2;
-                    int bj;
-                    double bd2;
-                    decide64(d, sc, vv, M, cand, nc, bj, bd2);
-                    d.pi[vv] = bj;
-                    d.d64[vv] = __dsqrt_rn(bd2);
-                }
-            }
-        }
-        __syncthreads();  // s_c / s_s are free again
-    }
+    const float sn = sqrtf(c1) / nrm * 1.00001f + 2.0f * assoc_band(M);
+    if (!(sn < 0.70710678f)) return INFINITY;
+    const float cs = sqrtf(1.0f - sn * sn);
+    return sn * sqrtf(2.0f / (1.0f + cs)) * 1.00001f + assoc_margin(M);
 }
 
-// Points whose FP32 band holds three or more references: one warp per point
-// re-evaluates, in FP64, every reference of the scanned angular range whose
-// FP32 distance lies within the band of the range minimum.
-__global__ void __launch_bounds__(256) k_rescan(Plan* plan)
+constexpr int kAssocWarps = 8;
+constexpr int kAssocFill = 2432;  // warps that keep the GPU busy: 16 per SM
+constexpr int kAssocMany = 6;     // balls within the warp's reach from which each point is asked
+
+template <int M>
+__global__ void __launch_bounds__(kAssocWarps * 32) k_assoc(Plan* plan, int pfirst, int plast)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int p = 0; p < plan->nprob; ++p) {
+    constexpr int MP = (M + 3) / 4 * 4, V = MP / 4;
+    __shared__ float4 s_u[kAssocWarps][32 * V];
+    __shared__ float s_pt[kAssocWarps][M + 1][32];  // unit directions and bounds of the warp's points
+    __shared__ int s_first[kMaxBatch + 1];
+    __shared__ int s_share;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // lanes per point: enough warps for the GPU, at most a warp per point;
+    // tasks (warps' worth of points) before each problem
+    if (tid == 0) {
+        long long tot = 0;
+        auto count = [&](int p) {
+            const ProbDev& d = plan->p[p];
+            return d.in.mode == MODE_SELECT && d.in.m == M && ld_volatile(&d.sc->status) == 0 ? ld_volatile(&d.sc->nS) : 0;
+        };
+        for (int p = pfirst; p < plast; ++p) tot += count(p);
+        int share = 1;
+        while (share < 32 && tot * share < (long long)kAssocFill * 32) share *= 2;
+        int acc = 0;
+        for (int p = pfirst; p < plast; ++p) {
+            s_first[p - pfirst] = acc;
+            acc += (int)cdiv(count(p), 32 / share);
+        }
+        s_first[plast - pfirst] = acc;
+        s_share = share;
+    }
+    __syncthreads();
+    const int share = s_share, ppw = 32 / share, sub = lane & (share - 1), ntask = s_first[plast - pfirst];
+    float4* const su = s_u[warp];
+    float (*const sp)[32] = s_pt[warp];
+    // a population split over GPUs associates only its own points
+    const bool ranged = plan->split.kind == SPLIT_ASSOC;
+    int p = pfirst;
+    for (;;) {
+        int task = 0;
+        if (lane == 0) task = (int)atomicAdd(&plan->asc_next[M], 1ull);
+        task = __shfl_sync(0xffffffffu, task, 0);
+        if (task >= ntask) break;
+        while (s_first[p + 1 - pfirst] <= task) ++p;
         const ProbDev& d = plan->p[p];
-        Scal* sc = d.sc;
-        if (d.in.mode != MODE_SELECT || ld_volatile(&sc->status) != 0) continue;
-        const int nflag = ld_volatile(&sc->nflag);
-        const int m = d.in.m, nr = d.in.n_r;
-        const int32_t* ro = d.rord + (int64_t)sc->rbuf * nr;
-        const float band = assoc_band(m);
-        for (int64_t w = gw; w < nflag; w += nw) {
-            const int64_t v = d.flagged[w];
-            const float bound = d.flagged_bound[w];
-            float f[kMaxM];
-            float n2 = 0.0f;
-            for (int k = 0; k < m; ++k) {
-                f[k] = (d.in.F[v * m + k] - sc->z[k]) * sc->inv_a32[k];
-                n2 = fmaf(f[k], f[k], n2);
+        Scal* const sc = d.sc;
+        const int nS = ld_volatile(&sc->nS), nr = d.in.n_r, nleaf = d.nrleaf, nnode = d.nrnode;
+        const int ls = d.nrleafp, ns = d.nrnodep;
+        const float* __restrict__ lball = d.rball;
+        const float* __restrict__ lrad = d.rrad;
+        const float* __restrict__ nball = d.rnball;
+        const float* __restrict__ nrad = d.rnrad;
+        const float4* __restrict__ rs = reinterpret_cast<const float4*>(d.rsort);
+        const int32_t* __restrict__ ro = d.rord;
+        const int64_t lo = ranged ? plan->split.col_lo : 0, hi = ranged ? plan->split.col_hi : d.in.n2;
+        const int s = (task - s_first[p - pfirst]) * ppw + lane / share;
+        const int64_t v = s < nS ? (int64_t)d.sord[s] : -1;
+        const bool act = v >= lo && v < hi && s < nS;
+        if (sub == 0 && s < nS) d.scell[s] = 0xffffffffu;  // candidates: none yet
+        float f[M], n2 = 0.0f;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            f[k] = act ? (d.in.F[v * M + k] - sc->z[k]) * sc->inv_a32[k] : 0.0f;
+            n2 = fmaf(f[k], f[k], n2);
+        }
+        const float nrm = sqrtf(n2);
+        const bool bad = act && (!(nrm > 0.0f) || !isfinite(nrm));
+        if (bad && sub == 0) {  // at the ideal point (or overflow): every reference in FP64
+            atomicAdd(&sc->nflag, 1);
+            d.flagged[atomicAdd(&sc->nbad, 1)] = (int32_t)v;
+        }
+        const bool seek = act && !bad;
+        const unsigned seekers = __ballot_sync(0xffffffffu, seek);
+        if (!seekers) continue;
+        // unit directions, their mean and the ball around it
+        float u[M], wc[M];
+        const float inv = seek ? 1.0f / nrm : 0.0f, part = 1.0f / (float)__popc(seekers);
+        float wr = 0.0f;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            u[k] = f[k] * inv;
+            float t = u[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            wc[k] = t * part;
+            const float e = u[k] - wc[k];
+            wr = fmaf(e, e, wr);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < M; ++k) sp[k][lane] = u[k];
+        wr = sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, seek ? __float_as_uint(wr) : 0u))) * 1.00001f + 1e-6f;
+
+        Top3 top;
+        top.init();
+        float chord = INFINITY, reach = INFINITY;  // the lane's bound; the warp's largest
+        auto stage = [&](int t) {                  // the 32 references of leaf t into shared memory
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < V; ++e) su[e * 32 + lane] = __ldg(&rs[(int64_t)t * 32 * V + e * 32 + lane]);
+            __syncwarp();
+        };
+        auto member = [&](int j, float (&r)[MP]) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const float4 x = su[j * V + e];
+                r[4 * e] = x.x; r[4 * e + 1] = x.y; r[4 * e + 2] = x.z; r[4 * e + 3] = x.w;
             }
-            const float nrm = sqrtf(n2);
-            // bad: at the ideal point or overflowed, every reference in FP64;
-            // otherwise the FP32 band of the range minimum filters the range
-            const bool bad = !(nrm > 0.0f) || !isfinite(nrm);
-            const bool all = bad || !(bound < INFINITY);
-            int lo = 0, hi = nr;
-            if (!all) {
-                const float phif = polar_angle(f, m);
-                lo = lower_bound_f(d.rphi, nr, phif - bound);
-                hi = lower_bound_f(d.rphi, nr, nextafterf(phif + bound, INFINITY));
+        };
+        // distance of a ball from the warp's, less both radii: at most the
+        // distance of any member from any of the points
+        auto gap = [&](const float* ball, const float* rad, int stride, int at) {
+            float d2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                const float e = __ldg(&ball[k * stride + at]) - wc[k];
+                d2 = fmaf(e, e, d2);
             }
-            auto dist32 = [&](int q) {
-                const float* u = d.rsort + (int64_t)q * m;
-                float g = f[0] * u[0];
-                for (int k = 1; k < m; ++k) g = fmaf(f[k], u[k], g);
+            return sqrtf(d2) * (1.0f - 1e-5f) - __ldg(&rad[at]) - wr;
+        };
+        auto nearest = [&](const float* ball, const float* rad, int stride, int from, int to) {  // by gap
+            float bg = INFINITY;
+            int bi = from;
+            for (int a = from + lane; a < to; a += 32) {
+                const float x = gap(ball, rad, stride, a);
+                if (x < bg) { bg = x; bi = a; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float og = __shfl_xor_sync(0xffffffffu, bg, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (og < bg || (og == bg && oi < bi)) { bg = og; bi = oi; }
+            }
+            return bi;
+        };
+        // whether one of the points may need ball `at` (a lane per ball, one
+        // point after the other)
+        auto wanted = [&](const float* ball, const float* rad, int stride, int at) {
+            float c[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) c[k] = __ldg(&ball[k * stride + at]);
+            const float r = __ldg(&rad[at]);
+            bool any = false;
+            for (unsigned left = seekers; left; left &= left - 1) {
+                const int i = __ffs(left) - 1;
+                if (i & (share - 1)) continue;
                 float d2 = 0.0f;
-                for (int k = 0; k < m; ++k) {
-                    const float e = fmaf(-g, u[k], f[k]);
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    const float e = c[k] - sp[k][i];
                     d2 = fmaf(e, e, d2);
                 }
-                return sqrtf(d2);
-            };
-            float dmin = INFINITY;
-            if (!bad)
-                for (int q = lo + lane; q < hi; q += 32) dmin = fminf(dmin, dist32(q));
+                const float lim = r + sp[M][i];
+                any = any || !(d2 > lim * lim);
+            }
+            return any;
+        };
+        const int an = nearest(nball, nrad, ns, 0, nnode);
+        const int first = nearest(lball, lrad, ls, an * 32, min(nleaf, an * 32 + 32));
+        // first leaf, then the nodes and leaves within reach
+        int b0 = -32, a = 0;
+        unsigned nodes = 0u, leaves = 0u;
+        for (int t = first;;) {
+            stage(t);
+            const int cnt = min(32, nr - t * 32);
+            for (int j = sub; j < cnt; j += share) {
+                float r[MP];
+                member(j, r);
+                top.add(d2_f32<M>(f, r), t * 32 + j);
+            }
+            float c = top.c1;
+            for (int o = 1; o < share; o <<= 1) c = fminf(c, __shfl_xor_sync(0xffffffffu, c, o));
+            chord = seek ? assoc_chord<M>(c, nrm) : 0.0f;
+            reach = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(chord)));
+            sp[M][lane] = chord;
+            __syncwarp();
+            // the next leaf that one of the points may need
+            t = -1;
+            while (t < 0) {
+                if (leaves) {
+                    const int c0 = a * 32 + __ffs(leaves) - 1;
+                    leaves &= leaves - 1;
+                    if (c0 == first) continue;
+                    float d2 = 0.0f;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dmin = fminf(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
-            const float lim = dmin + band * nrm;
-            double fn[kMaxM];
-            for (int k = 0; k < m; ++k) fn[k] = fnorm64(d.in.F[v * m + k], sc->z[k], sc->a[k]);
+                    for (int k = 0; k < M; ++k) {
+                        const float e = __ldg(&lball[k * ls + c0]) - u[k];
+                        d2 = fmaf(e, e, d2);
+                    }
+                    const float lim = __ldg(&lrad[c0]) + chord;
+                    if (__any_sync(0xffffffffu, seek && !(d2 > lim * lim))) t = c0;
+                } else if (nodes) {
+                    a = b0 + __ffs(nodes) - 1;
+                    nodes &= nodes - 1;
+                    const int c0 = a * 32 + lane;
+                    bool in = c0 < nleaf && !(gap(lball, lrad, ls, min(c0, nleaf - 1)) > reach);
+                    leaves = __ballot_sync(0xffffffffu, in);
+                    if (__popc(leaves) >= kAssocMany) {
+                        in = in && wanted(lball, lrad, ls, min(c0, nleaf - 1));
+                        leaves = __ballot_sync(0xffffffffu, in);
+                    }
+                } else {
+                    b0 += 32;
+                    if (b0 >= nnode) break;
+                    const int a0 = min(b0 + lane, nnode - 1);
+                    bool in = b0 + lane < nnode && !(gap(nball, nrad, ns, a0) > reach);
+                    nodes = __ballot_sync(0xffffffffu, in);
+                    if (__popc(nodes) >= kAssocMany) {
+                        in = in && wanted(nball, nrad, ns, a0);
+                        nodes = __ballot_sync(0xffffffffu, in);
+                    }
+                }
+            }
+            if (t < 0) break;
+        }
+        // the lanes that share a point merge their lists
+        for (int o = 1; o < share; o <<= 1) {
+            const float e1 = __shfl_xor_sync(0xffffffffu, top.c1, o), e2 = __shfl_xor_sync(0xffffffffu, top.c2, o),
+                        e3 = __shfl_xor_sync(0xffffffffu, top.c3, o);
+            const int i1 = __shfl_xor_sync(0xffffffffu, top.s1, o), i2 = __shfl_xor_sync(0xffffffffu, top.s2, o);
+            top.add(e1, i1);
+            top.add(e2, i2);
+            top.add(e3, -1);
+        }
+        const float lim = sqrtf(top.c1) + assoc_band(M) * nrm;
+        const bool mine = seek && sub == 0;
+        const bool three = mine && sqrtf(top.c3) <= lim;  // three or more references inside the band
+        if (mine && !three) {  // one or two candidates for the FP64 decision
+            d.scell[s] = (uint32_t)__ldg(&ro[top.s1]);
+            d.sslot[s] = top.s2 >= 0 && sqrtf(top.c2) <= lim ? (uint32_t)__ldg(&ro[top.s2]) : 0xffffffffu;
+        }
+        // those points, one after the other: a lane per reference, the ones
+        // inside the band in FP64
+        for (unsigned left = __ballot_sync(0xffffffffu, three); left; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int64_t pv = __shfl_sync(0xffffffffu, (int)v, src);
+            const float plim = __shfl_sync(0xffffffffu, lim, src);
+            const float pchord = __shfl_sync(0xffffffffu, assoc_chord<M>(top.c1, nrm), src);
+            float pf[M], pu[M];
+            double fn[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                pf[k] = __shfl_sync(0xffffffffu, f[k], src);
+                pu[k] = __shfl_sync(0xffffffffu, u[k], src);
+                fn[k] = fnorm64(d.in.F[pv * M + k], sc->z[k], sc->a[k]);
+            }
             double bd2 = INFINITY;
             int bj = INT32_MAX;
-            for (int q = lo + lane; q < hi; q += 32) {
-                if (bad || dist32(q) <= lim) {
-                    const int j = __ldg(&ro[q]);
-                    const double d2 = perp_d2(fn, d.in.R + (int64_t)j * m, m);
-                    if (d2 < bd2 || (d2 == bd2 && j < bj)) { bd2 = d2; bj = j; }
+            auto near = [&](const float* ball, const float* rad, int stride, int at) {
+                float d2 = 0.0f;
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    const float e = __ldg(&ball[k * stride + at]) - pu[k];
+                    d2 = fmaf(e, e, d2);
+                }
+                const float r = __ldg(&rad[at]) + pchord;
+                return !(d2 > r * r);
+            };
+            for (int a0 = 0; a0 < nnode; a0 += 32) {
+                unsigned an2 = __ballot_sync(0xffffffffu, a0 + lane < nnode && near(nball, nrad, ns, min(a0 + lane, nnode - 1)));
+                for (; an2; an2 &= an2 - 1) {
+                    const int c0 = (a0 + __ffs(an2) - 1) * 32;
+                    unsigned lf = __ballot_sync(0xffffffffu, c0 + lane < nleaf && near(lball, lrad, ls, min(c0 + lane, nleaf - 1)));
+                    for (; lf; lf &= lf - 1) {
+                        const int t = c0 + __ffs(lf) - 1;
+                        stage(t);
+                        float r[MP];
+                        member(lane, r);
+                        if (t * 32 + lane < nr && sqrtf(d2_f32<M>(pf, r)) <= plim) {
+                            const int j = __ldg(&ro[t * 32 + lane]);
+                            const double d2 = perp_d2(fn, d.in.R + (int64_t)j * M, M);
+                            if (d2 < bd2 || (d2 == bd2 && j < bj)) { bd2 = d2; bj = j; }
+                        }
+                    }
                 }
             }
 #pragma unroll
@@ -693,13 +675,90 @@ __global__ void __launch_bounds__(256) k_rescan(Plan* plan)
                 if (od < bd2 || (od == bd2 && oj < bj)) { bd2 = od; bj = oj; }
             }
             if (lane == 0) {
+                atomicAdd(&sc->nflag, 1);
                 if (bj == INT32_MAX) {  // every distance was NaN
                     set_status(sc, EMO_ERR_NONFINITE);
                     bj = 0;
                 }
-                d.pi[v] = bj;
-                d.d64[v] = __dsqrt_rn(bd2);
+                d.pi[pv] = bj;
+                d.d64[pv] = __dsqrt_rn(bd2);
             }
+        }
+    }
+}
+
+// The FP64 decision between the candidates of each point (a thread per point:
+// with several lanes to a point in the search, FP64 there would run mostly
+// empty warps), and the points at the ideal point or whose normalised
+// objectives overflow, where a warp evaluates every reference. Bound by FP64:
+// four divisions and a square root per point.
+template <int MM>
+__device__ __forceinline__ void decide_points(const ProbDev& d, int64_t first, int64_t stride)
+{
+    Scal* const sc = d.sc;
+    const int m = MM == kMaxM ? d.in.m : MM;
+    const int nS = ld_volatile(&sc->nS);
+    double z[MM], a[MM];
+#pragma unroll
+    for (int k = 0; k < MM; ++k)
+        if (k < m) { z[k] = (double)sc->z[k]; a[k] = sc->a[k]; }
+    for (int64_t s = first; s < nS; s += stride) {
+        const int j1 = (int)d.scell[s];
+        if (j1 < 0) continue;  // associated by the search, or listed
+        const int j2 = (int)d.sslot[s];
+        const int64_t v = d.sord[s];
+        double fn[MM];
+#pragma unroll
+        for (int k = 0; k < MM; ++k)
+            if (k < m) fn[k] = __ddiv_rn(__dsub_rn((double)d.in.F[v * m + k], z[k]), a[k]);
+        int bj = j1;
+        double bd2 = perp_d2(fn, d.in.R + (int64_t)j1 * m, m);
+        if (j2 >= 0) {
+            const double d2 = perp_d2(fn, d.in.R + (int64_t)j2 * m, m);
+            if (d2 < bd2 || (d2 == bd2 && j2 < bj)) { bd2 = d2; bj = j2; }
+        }
+        d.pi[v] = bj;
+        d.d64[v] = __dsqrt_rn(bd2);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_decide(Plan* plan)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    const ProbDev& d = plan->p[blockIdx.y];
+    Scal* sc = d.sc;
+    if (d.in.mode != MODE_SELECT || ld_volatile(&sc->status) != 0) return;
+    const int m = d.in.m, nr = d.in.n_r;
+    switch (m) {
+    case 2: decide_points<2>(d, t0, stride); break;
+    case 3: decide_points<3>(d, t0, stride); break;
+    default: decide_points<kMaxM>(d, t0, stride);
+    }
+    const int nbad = ld_volatile(&sc->nbad);
+    for (int64_t w = t0 >> 5; w < nbad; w += stride >> 5) {
+        const int64_t v = d.flagged[w];
+        double fn[kMaxM];
+        for (int k = 0; k < m; ++k) fn[k] = fnorm64(d.in.F[v * m + k], sc->z[k], sc->a[k]);
+        double bd2 = INFINITY;
+        int bj = INT32_MAX;
+        for (int j = lane; j < nr; j += 32) {
+            const double d2 = perp_d2(fn, d.in.R + (int64_t)j * m, m);
+            if (d2 < bd2 || (d2 == bd2 && j < bj)) { bd2 = d2; bj = j; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double od = __shfl_xor_sync(0xffffffffu, bd2, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+            if (od < bd2 || (od == bd2 && oj < bj)) { bd2 = od; bj = oj; }
+        }
+        if (lane == 0) {
+            if (bj == INT32_MAX) {  // every distance was NaN
+                set_status(sc, EMO_ERR_NONFINITE);
+                bj = 0;
+            }
+            d.pi[v] = bj;
+            d.d64[v] = __dsqrt_rn(bd2);
         }
     }
 }
@@ -711,16 +770,11 @@ cudaError_t launch_assoc(Plan* plan, int nprob, const int* m_of, int sms, int bl
         int q = p;
         while (q < nprob && m_of[q] == m_of[p]) ++q;
         const unsigned grid = (unsigned)sms * (unsigned)(blocks_per_sm > 0 ? blocks_per_sm : 8);
-        // m >= 4: every reference, tiled (tiles from a counter: a few CTAs per SM)
-        const unsigned grid_all = (unsigned)sms * 4u;
         switch (m_of[p]) {
 #define X(MM) \
-    case MM: k_assoc_m<MM><<<grid, 256, 0, s>>>(plan, p, q); break;
-#define Y(MM) \
-    case MM: k_assoc_all<MM><<<grid_all, kBfWarps * 32, 0, s>>>(plan, p, q); break;
-            X(2) X(3) Y(4) Y(5) Y(6) Y(7) Y(8) Y(9) Y(10) Y(11) Y(12) Y(13) Y(14) Y(15) Y(16)
+    case MM: k_assoc<MM><<<grid, kAssocWarps * 32, 0, s>>>(plan, p, q); break;
+            X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
 #undef X
-#undef Y
         default: return cudaErrorInvalidValue;
         }
         cudaError_t e = cudaGetLastError();
