@@ -85,6 +85,7 @@ long long spin_budget()
 }
 
 struct DevInfo {
+    int32_t* sticky = nullptr;  // address of the sticky device status
     int sms = 0;
     int G = 0;  // CTAs of each cooperative launch
     bool ok = false;
@@ -129,6 +130,8 @@ DevInfo dev_info()
             occ = std::min(occ, o);
         }
         if (occ < 1) return DevInfo{};
+        di.sticky = sticky_address();
+        if (!di.sticky) return DevInfo{};
         di.sms = sms;
         di.G = sms * occ;
         di.ok = true;
@@ -603,6 +606,7 @@ emo_status emo_moead_select(const float* X, const float* F1, const float* O, con
     if ((int64_t)ws_bytes < moead_layout(n, m, T, (char*)ws, &a)) return EMO_ERR_WORKSPACE;
     DevInfo di = dev_info();
     if (!di.ok) return EMO_ERR_CUDA;
+    a.sticky = di.sticky;
     a.X = X;
     a.F1 = F1;
     a.O = O;

@@ -12,12 +12,12 @@ cudaError_t launch_assoc(Plan* plan, int nprob, const int* m_of, int sms, int bl
 // Sticky device status: the first failure any call on this device reported
 // since the last read (k_finish sets it); read after the stream's prior work.
 cudaError_t sticky_status(cudaStream_t s, int32_t* out, bool clear);
-// Folds a call's device status word into the sticky status (stream order).
-cudaError_t sticky_merge(const int32_t* status, cudaStream_t s);
+// Its address on the current device (null on an error).
+int32_t* sticky_address();
 
 // TensorMOEA/D selection (Algorithm S.8): caller arrays and the workspace
 // regions (status word, z_min keys, per-subproblem best marked value and
-// its lowest offspring index, per-pair marked value).
+// its lowest offspring index, the pairs decided in FP64, the filter's records).
 struct MoeadArgs {
     const float* X;
     const float* F1;
@@ -34,12 +34,18 @@ struct MoeadArgs {
     int32_t m, T;
     double theta;
     int32_t* status;
+    int32_t* sticky;  // sticky device status
     uint32_t* zkey;
     unsigned long long* gmin;
     int32_t* tie;
-    double* gpair;
-    double* sub;  // [n][m + 2]: ||w_j||, the subproblem's own PBI value, w_j / ||w_j||
+    double* gpair;               // [n T] every pair's marked value, where no records fit
+    uint32_t* exact;             // [n T] pairs decided in FP64 that mark their subproblem
+    unsigned long long* nexact;  // how many
+    double* sub;                 // [n][m + 2]: ||w_j||, the subproblem's own PBI value, w_j / ||w_j||
+    float* rec;                  // [n][moead_rec(m)]: w_j / ||w_j|| and the own value rounded up, in float (nullable)
 };
+// Floats of a record: m + 1, rounded up to whole float4.
+__host__ __device__ constexpr int moead_rec(int m) { return (m + 4) / 4 * 4; }
 // Workspace bytes of one TensorMOEA/D selection (regions 256-byte aligned);
 // fills the region pointers of `a` when `ws` is given.
 int64_t moead_layout(int64_t n, int32_t m, int32_t T, char* ws, MoeadArgs* a);
