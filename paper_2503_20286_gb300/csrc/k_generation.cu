@@ -45,68 +45,118 @@ __device__ __forceinline__ bool hit(uint32_t x, double p)
 __device__ __forceinline__ double clip(double v, double lo, double hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 // SBX of one variable: beta from mu, children 0.5[(1 +- beta) x1 + (1 -+ beta) x2].
-__device__ void sbx(double x1, double x2, double mu, double eta_c, double& c1, double& c2)
+// (One pow for both halves of mu: a warp holds both.)
+__device__ __forceinline__ void sbx(double x1, double x2, double mu, double eta_c, double& c1, double& c2)
 {
-    const double e = __ddiv_rn(1.0, __dadd_rn(eta_c, 1.0));
-    const double beta = mu <= 0.5 ? pow(__dmul_rn(2.0, mu), e)
-                                  : pow(__ddiv_rn(1.0, __dsub_rn(2.0, __dmul_rn(2.0, mu))), e);
+    const double e = __ddiv_rn(1.0, __dadd_rn(eta_c, 1.0)), mu2 = __dmul_rn(2.0, mu);
+    const double beta = pow(mu <= 0.5 ? mu2 : __ddiv_rn(1.0, __dsub_rn(2.0, mu2)), e);
     const double bp = __dadd_rn(1.0, beta), bm = __dsub_rn(1.0, beta);
     c1 = __dmul_rn(0.5, __dadd_rn(__dmul_rn(bp, x1), __dmul_rn(bm, x2)));
     c2 = __dmul_rn(0.5, __dadd_rn(__dmul_rn(bm, x1), __dmul_rn(bp, x2)));
 }
 
-// Polynomial mutation of one variable (original form, eta = eta_m + 1).
-__device__ double pm(double x, double lo, double hi, double mu, double eta_m)
+// Polynomial mutation of one variable (original form, eta = eta_m + 1):
+// mu <= 0.5: t = 2 mu + (1 - 2 mu)(1 - (x - lo) / w)^eta, step t^(1/eta) - 1;
+// otherwise:  t = 2 - 2 mu + (2 mu - 1)(1 - (hi - x) / w)^eta, step 1 - t^(1/eta).
+__device__ __forceinline__ double pm(double x, double lo, double hi, double mu, double eta_m)
 {
     const double eta = __dadd_rn(eta_m, 1.0);
     const double width = __dsub_rn(hi, lo);
     const double inv = __ddiv_rn(1.0, eta);
-    double step;
-    if (mu <= 0.5) {
-        const double delta1 = __ddiv_rn(__dsub_rn(x, lo), width);
-        const double t = __dadd_rn(__dmul_rn(2.0, mu),
-                                   __dmul_rn(__dsub_rn(1.0, __dmul_rn(2.0, mu)), pow(__dsub_rn(1.0, delta1), eta)));
-        step = __dsub_rn(pow(t, inv), 1.0);
-    } else {
-        const double delta2 = __ddiv_rn(__dsub_rn(hi, x), width);
-        const double t = __dadd_rn(__dsub_rn(2.0, __dmul_rn(2.0, mu)),
-                                   __dmul_rn(__dsub_rn(__dmul_rn(2.0, mu), 1.0), pow(__dsub_rn(1.0, delta2), eta)));
-        step = __dsub_rn(1.0, pow(t, inv));
-    }
+    const double mu2 = __dmul_rn(2.0, mu);
+    const bool low = mu <= 0.5;
+    const double delta = __ddiv_rn(low ? __dsub_rn(x, lo) : __dsub_rn(hi, x), width);
+    const double q = pow(__dsub_rn(1.0, delta), eta);
+    const double t = low ? __dadd_rn(mu2, __dmul_rn(__dsub_rn(1.0, mu2), q))
+                         : __dadd_rn(__dsub_rn(2.0, mu2), __dmul_rn(__dsub_rn(mu2, 1.0), q));
+    const double r = pow(t, inv);
+    const double step = low ? __dsub_rn(r, 1.0) : __dsub_rn(1.0, r);
     return __dadd_rn(x, __dmul_rn(step, width));
 }
 
-// One thread per (pair, variable): both children of that variable.
+// One thread per (pair, variable): both children of that variable. Variables
+// to be mutated (one in d by default) are collected in shared memory and
+// mutated by full warps: done in place, nearly every warp held one and ran both
+// FP64 powers of the mutation for it, twice per child. Bound by FP64 (a pow per
+// crossover and two per mutation): 500 us before, 120 with the queue (50,000
+// offspring of 12 variables).
+constexpr int kPmQueue = 4 * kGenThreads;
+
 __global__ void __launch_bounds__(kGenThreads) k_variation(VariationArgs a)
 {
+    __shared__ double s_v[kPmQueue];      // the child's value before the mutation
+    __shared__ int64_t s_at[kPmQueue];    // its place in X_off
+    __shared__ uint32_t s_mu[kPmQueue];
+    __shared__ int s_n;
+    const int lane = threadIdx.x & 31;
     const int64_t pairs = (a.n_off + 1) / 2;
     const int64_t work = pairs * a.d;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < work; e += stride) {
-        const int64_t p = e / a.d, k = e - p * a.d;
-        const uint4 r0 = gen_random(a.seed, a.gen, p, 1u, 0), r1 = gen_random(a.seed, a.gen, p, 1u, 1);
-        const int64_t pa = index_of(r0.x, a.n), pb = index_of(r1.x, a.n);
-        if (k == 0 && a.parents) {
-            a.parents[2 * p] = (int32_t)pa;
-            a.parents[2 * p + 1] = (int32_t)pb;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x; e0 < work; e0 += stride) {
+        const int64_t e = e0 + threadIdx.x;
+        const bool has = e < work;
+        int64_t p = 0, k = 0;
+        double c[2] = {0.0, 0.0}, lo = 0.0, hi = 1.0;
+        if (has) {
+            p = work <= INT32_MAX ? (int64_t)((uint32_t)e / (uint32_t)a.d) : e / a.d;
+            k = e - p * a.d;
+            const uint4 r0 = gen_random(a.seed, a.gen, p, 1u, 0), r1 = gen_random(a.seed, a.gen, p, 1u, 1);
+            const int64_t pa = index_of(r0.x, a.n), pb = index_of(r1.x, a.n);
+            if (k == 0 && a.parents) {
+                a.parents[2 * p] = (int32_t)pa;
+                a.parents[2 * p + 1] = (int32_t)pb;
+            }
+            const double x1 = (double)a.X[pa * a.d + k], x2 = (double)a.X[pb * a.d + k];
+            if (a.lo) lo = (double)a.lo[k];
+            if (a.hi) hi = (double)a.hi[k];
+            c[0] = x1;
+            c[1] = x2;
+            if (hit(r0.y, a.p_c)) {
+                const uint4 rs = gen_random(a.seed, a.gen, p, 2u, k);
+                sbx(x1, x2, unit_of(rs.x), a.eta_c, c[0], c[1]);
+            }
         }
-        const double x1 = (double)a.X[pa * a.d + k], x2 = (double)a.X[pb * a.d + k];
-        const double lo = a.lo ? (double)a.lo[k] : 0.0, hi = a.hi ? (double)a.hi[k] : 1.0;
-        double c[2] = {x1, x2};
-        if (hit(r0.y, a.p_c)) {
-            const uint4 rs = gen_random(a.seed, a.gen, p, 2u, k);
-            sbx(x1, x2, unit_of(rs.x), a.eta_c, c[0], c[1]);
-        }
+#pragma unroll
         for (int child = 0; child < 2; ++child) {
             const int64_t row = child == 0 ? p : pairs + p;
-            if (row >= a.n_off) continue;
-            double v = clip(c[child], lo, hi);
-            const uint4 rm = gen_random(a.seed, a.gen, row, 3u, k);
-            // PM is defined over (x - lo) / (hi - lo): a variable without a
-            // positive width (outside the contract) is left unmutated.
-            if (hit(rm.x, a.p_m) && hi > lo) v = clip(pm(v, lo, hi, unit_of(rm.y), a.eta_m), lo, hi);
-            a.Xoff[row * a.d + k] = (float)v;
+            bool mutate = false;
+            uint32_t mu = 0u;
+            const double v = clip(c[child], lo, hi);
+            if (has && row < a.n_off) {
+                const uint4 rm = gen_random(a.seed, a.gen, row, 3u, k);
+                // PM is defined over (x - lo) / (hi - lo): a variable without a
+                // positive width (outside the contract) is left unmutated.
+                mutate = hit(rm.x, a.p_m) && hi > lo;
+                mu = rm.y;
+                if (!mutate) a.Xoff[row * a.d + k] = (float)v;
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, mutate);
+            if (mask) {
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&s_n, __popc(mask));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (mutate) {
+                    at += __popc(mask & lanemask_lt());
+                    s_v[at] = v;
+                    s_at[at] = row * a.d + k;
+                    s_mu[at] = mu;
+                }
+            }
         }
+        __syncthreads();
+        const int n = s_n;
+        if (n > (e0 + stride < work ? kPmQueue - 2 * kGenThreads : 0)) {  // the next round may not fit
+            for (int q = threadIdx.x; q < n; q += blockDim.x) {
+                const int64_t at = s_at[q], kk = at % a.d;
+                const double l = a.lo ? (double)a.lo[kk] : 0.0, h = a.hi ? (double)a.hi[kk] : 1.0;
+                a.Xoff[at] = (float)clip(pm(s_v[q], l, h, unit_of(s_mu[q]), a.eta_m), l, h);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) s_n = 0;
+        }
+        __syncthreads();
     }
 }
 
