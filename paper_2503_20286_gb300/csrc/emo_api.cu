@@ -164,15 +164,27 @@ ProbIn make_in(const float* F, const float* R, int64_t n2, int32_t m, int32_t n_
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
+// A cooperative kernel on the CTAs that its groups use; a single CTA waits for
+// nobody and needs no cooperative launch.
+cudaError_t launch_group(const void* fn, int ctas, int threads, size_t smem, cudaStream_t s, void** args)
+{
+    if (ctas == 1) return cudaLaunchKernel(fn, dim3(1), dim3(threads), args, smem, s);
+    return cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(threads), args, smem, s);
+}
 cudaError_t coop(const void* fn, int G, size_t smem, cudaStream_t s, Plan* plan, int threads = kCoopThreads)
 {
     void* args[] = {&plan};
-    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(threads), args, smem, s);
+    return launch_group(fn, G, threads, smem, s, args);
 }
 cudaError_t coop_phase(const void* fn, int G, size_t smem, cudaStream_t s, Plan* plan, int phase)
 {
     void* args[] = {&plan, &phase};
-    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kCoopThreads), args, smem, s);
+    return launch_group(fn, G, kCoopThreads, smem, s, args);
+}
+// CTAs of one kind of group over all problems (a batch fills the grid).
+int group_ctas(GroupKind kind, const std::vector<ProbIn>& ins, int G)
+{
+    return ins.size() == 1 ? group_cap(kind, ins[0], G) : G;
 }
 
 // Launch shapes, per (compute capability as 10 * major + minor, m,
@@ -262,13 +274,13 @@ emo_status run_niche_stages(std::vector<ProbIn>& ins, const DevInfo& di, Plan* p
 emo_status run_selection_stages(std::vector<ProbIn>& ins, const DevInfo& di, Plan* plan, int dev, cudaStream_t s,
                                 StageMarker& sm, bool finish = true, int split = SPLIT_NONE)
 {
-    const int nprob = (int)ins.size();
+    const int nprob = (int)ins.size(), narrow = group_ctas(GRP_NARROW, ins, di.G);
     if (split == SPLIT_NICHE) {
-        if (coop((const void*)k_given_in, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+        if (coop((const void*)k_given_in, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("given");
         return run_niche_stages(ins, di, plan, s, sm, finish);
     }
-    if (coop((const void*)k_stats, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (coop((const void*)k_stats, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("stats");
     std::vector<int> m_of(nprob);
     for (int p = 0; p < nprob; ++p) m_of[p] = ins[p].m;
@@ -284,10 +296,10 @@ emo_status run_selection_stages(std::vector<ProbIn>& ins, const DevInfo& di, Pla
     if (cudaGetLastError() != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("rescan");
     if (split == SPLIT_ASSOC) {
-        if (coop((const void*)k_assoc_out, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+        if (coop((const void*)k_assoc_out, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("assoc_out");
         if (finish) {  // status and info
-            if (coop((const void*)k_finish, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+            if (coop((const void*)k_finish, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
             sm.mark("finish");
         }
         return EMO_OK;
@@ -299,18 +311,19 @@ emo_status run_selection_stages(std::vector<ProbIn>& ins, const DevInfo& di, Pla
 emo_status run_niche_stages(std::vector<ProbIn>& ins, const DevInfo& di, Plan* plan, cudaStream_t s,
                             StageMarker& sm, bool finish)
 {
-    if (coop((const void*)k_csr, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    const int narrow = group_ctas(GRP_NARROW, ins, di.G);
+    if (coop((const void*)k_csr, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("csr");
     bool any_exact = false, any_oneshot = false;
     for (const ProbIn& in : ins) {
         any_exact |= in.mode == MODE_SELECT && in.niche == EMO_NICHE_EXACT;
         any_oneshot |= in.mode == MODE_SELECT && in.niche == EMO_NICHE_ONESHOT;
     }
-    if (any_exact && coop((const void*)k_niche, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
-    if (any_oneshot && coop((const void*)k_niche_oneshot, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (any_exact && coop((const void*)k_niche, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (any_oneshot && coop((const void*)k_niche_oneshot, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("niche");
     if (finish) {
-        if (coop((const void*)k_finish, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+        if (coop((const void*)k_finish, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("finish");
     }
     return EMO_OK;
@@ -364,16 +377,18 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     Plan* plan = (Plan*)ws;
     char* base = (char*)ws;
 
+    const int narrow = group_ctas(GRP_NARROW, ins, di.G);
     StageMarker sm(s);
     k_setup<<<1, 128, 0, s>>>(args, sp, plan, base);
     if (cudaGetLastError() != cudaSuccess) return EMO_ERR_CUDA;
-    k_prep<<<dim3((unsigned)std::max(1, di.sms * 2 / nprob), nprob), 256, 0, s>>>(plan);
+    // (a batch's problems are uneven: up to 32 CTAs each, the small ones leave)
+    k_prep<<<dim3((unsigned)(nprob == 1 ? di.sms * 2 : std::max(di.sms * 2 / nprob, 32)), nprob), 256, 0, s>>>(plan);
     if (cudaGetLastError() != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("prep");
     // (from given ranks only the references are ordered; the niching from a
     // given association has none)
-    if (any_lex && coop((const void*)k_sort, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
-    if (sp.kind != SPLIT_NICHE && (any_tree || any_select) && coop((const void*)k_order, di.G, 0, s, plan) != cudaSuccess)
+    if (any_lex && coop((const void*)k_sort, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (sp.kind != SPLIT_NICHE && (any_tree || any_select) && coop((const void*)k_order, narrow, 0, s, plan) != cudaSuccess)
         return EMO_ERR_CUDA;
     sm.mark("sort");
     if (nprob == 1 && ins[0].mode == MODE_DOM) {  // caller-order dominance matrix only
@@ -383,12 +398,12 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
             return EMO_ERR_CUDA;
         sm.mark("dominance");
         // status word of the workspace and the sticky device status
-        if (coop((const void*)k_finish, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+        if (coop((const void*)k_finish, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("finish");
         return EMO_OK;
     }
     if (nprob == 1 && ins[0].ranked) {  // the ranks are given: no dominance matrix, no peeling
-        if (coop((const void*)k_rank_in, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+        if (coop((const void*)k_rank_in, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("rank_in");
         return run_selection_stages(ins, di, plan, dev, s, sm, true, sp.kind);
     }
@@ -419,7 +434,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         if (coop(wave ? (const void*)k_peel_wave : (const void*)k_peel, di.G, smem, s, plan) != cudaSuccess)
             return EMO_ERR_CUDA;
     }
-    if (any_tree && coop((const void*)k_fronts, di.G, (size_t)fronts_smem, s, plan, kTreeThreads) != cudaSuccess)
+    if (any_tree && coop((const void*)k_fronts, group_ctas(GRP_TREE, ins, di.G), (size_t)fronts_smem, s, plan, kTreeThreads) != cudaSuccess)
         return EMO_ERR_CUDA;
     sm.mark("peel");
     if (any_select) {
@@ -438,7 +453,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         if (coop_phase((const void*)k_hype, di.G, 0, s, plan, 1) != cudaSuccess) return EMO_ERR_CUDA;
         sm.mark("hype");
     }
-    if (coop((const void*)k_finish, di.G, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
+    if (coop((const void*)k_finish, narrow, 0, s, plan) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("finish");
     return EMO_OK;
 }

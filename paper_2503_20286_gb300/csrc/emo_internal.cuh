@@ -37,6 +37,7 @@ constexpr int kColBlock = 1024;       // columns per column block
 constexpr int kDomRowChunk = 1024;    // row blocks per dominance work item (largest; emo_dominance)
 constexpr int kDomChunkMin = 64;      // smallest row-block chunk of a selection's dominance items
 constexpr int kCoopThreads = 512;     // threads of the cooperative kernels
+constexpr int kOneCtaItems = 1024;    // points and references that one CTA serves alone
 constexpr int kNicheBins = 4096;      // niching select: bins of the top 12 bits of a priority
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
@@ -334,6 +335,31 @@ __host__ __device__ __forceinline__ int fronts_smem_bytes(int64_t n2, int m)
                  (nleaf < front_local(m) ? nleaf : front_local(m)) * (4 + 32 * (m + 1)) * 4);
 }
 
+// CTA groups of the cooperative kernels: wide (peeling from the matrix,
+// TensorHypE), tree (peeling by the z-order tree), narrow (the others).
+enum GroupKind : int { GRP_NARROW = 0, GRP_WIDE = 1, GRP_TREE = 2 };
+// Most CTAs that a problem's group gets out of G: its launch shapes' caps, and
+// no more than it can use. A barrier of two CTAs costs as much as one of 152
+// (1.1 us), none inside a single CTA, so small problems get one CTA: a
+// selection of 500 points on 250 directions takes 199 us so and 207 with the
+// narrow kernels on two CTAs; 16 leaves per CTA of the tree (ranking 600
+// points, 19 leaves: 126 us by one CTA, 109 by two; 1,000 points 162 and 129).
+__host__ __device__ __forceinline__ int group_cap(GroupKind kind, const ProbIn& in, int G)
+{
+    int64_t c = in.cap_wide > 0 && in.cap_wide < G ? in.cap_wide : G;
+    if (kind == GRP_NARROW) {
+        if (in.cap_narrow > 0 && in.cap_narrow < c) c = in.cap_narrow;
+        const int64_t items = in.n2 + (in.mode == MODE_SELECT ? in.n_r : 0);
+        const int64_t use = items <= kOneCtaItems ? 1 : cdiv(items, kCoopThreads);
+        if (use < c) c = use;
+    } else if (kind == GRP_TREE) {
+        const int64_t nleaf = cdiv(in.n2, 32);
+        const int64_t use = cdiv(nleaf, kTreeThreads / 64);
+        if (use < c) c = use;
+    }
+    return (int)c;
+}
+
 // Byte layout of one problem region; fills `d` when base != 0. Returns the
 // region size. The same function sizes the workspace on the host and carves
 // it on the device.
@@ -597,12 +623,9 @@ struct Group {
     int size;       // CTAs in the group
     unsigned* bar;  // the group's barrier counter (all kernels of one assignment use the same size)
 };
-// The group of this CTA in the wide (peeling from the matrix, TensorHypE),
-// the tree (peeling by the z-order tree) or the narrow (every other
-// cooperative kernel) assignment; prob = -1 for a CTA that serves no problem
-// (groups are capped by the problems' sizes and launch shapes), which returns
-// at once.
-enum GroupKind : int { GRP_NARROW = 0, GRP_WIDE = 1, GRP_TREE = 2 };
+// The group of this CTA in one of the assignments; prob = -1 for a CTA that
+// serves no problem (groups are capped by the problems' sizes and launch
+// shapes), which returns at once.
 __device__ __forceinline__ Group group_of(const Plan* plan, GroupKind kind)
 {
     const int32_t* first = kind == GRP_WIDE ? plan->grp_first : (kind == GRP_TREE ? plan->grpt_first : plan->grpn_first);

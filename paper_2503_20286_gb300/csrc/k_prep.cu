@@ -27,54 +27,106 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
         uint32_t* sc = reinterpret_cast<uint32_t*>(ws + a.in[p].ws_off);
         for (int i = t & 31; i < (int)(sizeof(Scal) / 4); i += 32) sc[i] = 0u;
     }
-    // CTA groups of each kind: shares of the grid in proportion to the work,
-    // at least one CTA for every problem that the kind serves and at most the
-    // problem's cap. Wide groups by n2^2 (dominance tiles read per front), tree
-    // groups by the searches to expect, narrow ones by n2. CTAs beyond the groups serve no problem.
-    if (t < 96 && (t & 31) == 0) {
+    // CTA groups of each kind (one warp per kind, a lane per problem): shares of
+    // the grid in proportion to the work, at least one CTA for every problem that
+    // the kind serves and at most the problem's cap. Wide groups by n2^2
+    // (dominance tiles read per front), narrow ones by n2, tree groups by the CTA
+    // time to expect: 0.09 us per point of two or three objectives, 0.19 of
+    // five. A tree group gets the CTAs that hold its leaves in shared memory
+    // before the rest is shared out, where the grid suffices for that (38,524
+    // points of two objectives: 18 us a front with the leaves in global memory,
+    // 13 in shared). CTAs beyond the groups serve no problem.
+    if (t < 96) {
+        __shared__ int s_cnt[3][kMaxBatch];
         const GroupKind kind = (GroupKind)(t >> 5);
-        auto weight = [&](int p) -> double {
+        const int lane = t & 31;
+        int* const cnt = s_cnt[kind];
+        auto weight = [&](int p) -> float {
             const ProbIn& in = a.in[p];
-            const double n = (double)in.n2;
-            if (kind == GRP_WIDE) return tree_ranked(in) && in.mode != MODE_HYPE ? 0.0 : n * n;
-            // (searches grow with m: 5 ms of CTA time for 20,000 points of three
-            // objectives, 16 ms for 40,000 of five)
-            if (kind == GRP_TREE) return tree_ranked(in) ? n * (in.m - 1) : 0.0;
+            const float n = (float)in.n2;
+            if (kind == GRP_WIDE) return tree_ranked(in) && in.mode != MODE_HYPE ? 0.0f : n * n;
+            if (kind == GRP_TREE) return tree_ranked(in) ? n * max(2, in.m - 1) : 0.0f;
             return n;
         };
-        auto cap = [&](int p) -> int {
-            const ProbIn& in = a.in[p];
-            int c = in.cap_wide > 0 ? min(in.cap_wide, a.G) : a.G;
-            if (kind == GRP_NARROW && in.cap_narrow > 0) c = min(c, in.cap_narrow);
-            if (kind == GRP_TREE) c = min(c, (int)max((int64_t)1, cdiv(cdiv(in.n2, 32), kTreeThreads / 64)));
-            return c;
+        auto cap = [&](int p) { return group_cap(kind, a.in[p], a.G); };
+        auto least = [&](int p, bool held) -> int {
+            if (!held || kind != GRP_TREE) return 1;
+            return min(cap(p), (int)cdiv(cdiv(a.in[p].n2, 32), front_local(a.in[p].m)));
         };
         int32_t* first = kind == GRP_WIDE ? plan->grp_first : (kind == GRP_TREE ? plan->grpt_first : plan->grpn_first);
-        double tot = 0.0;
-        int served = 0;
-        for (int p = 0; p < a.nprob; ++p) {
-            const double w = weight(p);
-            tot += w;
-            served += w > 0.0;
+        if (a.nprob == 1) {
+            if (lane == 0) {
+                first[0] = 0;
+                first[1] = weight(0) > 0.0f ? cap(0) : 0;
+            }
+        } else {
+            float tot = 0.0f;
+            int sum = 0;  // of the least numbers
+            for (int p = lane; p < a.nprob; p += 32) {
+                const float w = weight(p);
+                tot += w;
+                if (w > 0.0f) sum += least(p, true);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            const bool held = sum <= a.G;
+            // what a proportional share exceeds the least number by, scaled to a
+            // little less than what is left (so that no rounding takes it above)
+            const float unit = tot > 0.0f ? (float)a.G / tot : 0.0f;
+            float over = 0.0f;
+            sum = 0;
+            for (int p = lane; p < a.nprob; p += 32) {
+                const float w = weight(p);
+                if (w > 0.0f) {
+                    const int l = least(p, held);
+                    over += fmaxf(0.0f, w * unit - l);
+                    sum += l;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) over += __shfl_xor_sync(0xffffffffu, over, o);
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            const float scale = over > 0.0f ? (float)(a.G - sum) / over * 0.9999f : 0.0f;
+            int given = 0;
+            for (int p = lane; p < a.nprob; p += 32) {
+                const float w = weight(p);
+                cnt[p] = 0;
+                if (w > 0.0f) {
+                    const int l = least(p, held);
+                    cnt[p] = min(cap(p), l + (int)(fmaxf(0.0f, w * unit - l) * scale));
+                }
+                given += cnt[p];
+            }
+            given = __reduce_add_sync(0xffffffffu, given);
+            __syncwarp();
+            // the rest: one CTA each in turn to those below their cap
+            for (bool grew = true; given < a.G && grew;) {
+                grew = false;
+                for (int p0 = 0; p0 < a.nprob && given < a.G; p0 += 32) {
+                    const int p = p0 + lane;
+                    const bool can = p < a.nprob && cnt[p] > 0 && cnt[p] < cap(p);
+                    const unsigned ask = __ballot_sync(0xffffffffu, can);
+                    if (can && __popc(ask & ((1u << lane) - 1u)) < a.G - given) cnt[p]++;
+                    grew |= ask != 0u;
+                    given += min(__popc(ask), a.G - given);
+                }
+            }
+            __syncwarp();
+            int acc = 0;
+            for (int p0 = 0; p0 < a.nprob; p0 += 32) {
+                const int p = p0 + lane, c = p < a.nprob ? cnt[p] : 0;
+                int run = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, run, o);
+                    if (lane >= o) run += x;
+                }
+                if (p < a.nprob) first[p] = acc + run - c;
+                acc += __shfl_sync(0xffffffffu, run, 31);
+            }
+            if (lane == 0) first[a.nprob] = acc;
         }
-        const double per = tot > 0.0 ? (double)(a.G - served) / tot : 0.0;
-        int cnt[kMaxBatch], given = 0;
-        for (int p = 0; p < a.nprob; ++p) {
-            const double w = weight(p);
-            cnt[p] = w > 0.0 ? min(cap(p), 1 + (int)(w * per)) : 0;
-            given += cnt[p];
-        }
-        for (bool grew = true; given < a.G && grew;) {
-            grew = false;
-            for (int p = 0; p < a.nprob && given < a.G; ++p)
-                if (cnt[p] > 0 && cnt[p] < cap(p)) { cnt[p]++; given++; grew = true; }
-        }
-        int acc = 0;
-        for (int p = 0; p < a.nprob; ++p) {
-            first[p] = acc;
-            acc += cnt[p];
-        }
-        first[a.nprob] = acc;
     }
     if (t == 96) {
         plan->nprob = a.nprob;
@@ -94,16 +146,21 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
     }
 }
 
-// Validation and initialisation, grid (x, problem).
+// Validation and initialisation: as many CTAs per problem (a grid row each) as
+// its items need.
 __global__ void k_prep(Plan* plan)
 {
     const ProbDev& d = plan->p[blockIdx.y];
     const ProbIn& in = d.in;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t items = max(max(d.n2p, (int64_t)d.ncell), max((int64_t)in.n_r, 2 * (int64_t)d.nrcell));
+    const int64_t ctas = min((int64_t)gridDim.x, cdiv(items, blockDim.x)), stride = ctas * blockDim.x;
+    if ((int64_t)blockIdx.x >= ctas) return;
     const int64_t n2 = in.n2, m = in.m;
     bool bad = false;
-    if (in.F) {  // null only for the niching from a given association
+    if (in.F && !lex_ordered(in)) {
+        for (int64_t e = tid; e < n2 * m; e += stride) bad |= !isfinite(in.F[e]);
+    } else if (in.F) {  // null only for the niching from a given association
         // finiteness, and which bits of each objective's sort key vary (a
         // radix pass over a byte that no point changes is skipped)
         uint32_t kor[kMaxM], kinv[kMaxM];
