@@ -112,7 +112,7 @@ DevInfo dev_info()
             cudaFuncSetAttribute((const void*)k_fronts, cudaFuncAttributeMaxDynamicSharedMemorySize, kFrontsDynSmem) !=
                 cudaSuccess ||
             cudaFuncSetAttribute((const void*)k_hype_counts, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 hype_counts_smem(4)) != cudaSuccess)
+                                 hype_counts_smem(kSegKeys + 1)) != cudaSuccess)
             return DevInfo{};
         int occ = 2;
         // k_peel takes peel_smem_bytes(ncb) of dynamic shared memory, the others none
@@ -246,6 +246,28 @@ Shape default_shape(int sms, int64_t n2)
     return sh;
 }
 
+// Row blocks per item of the caller-order matrix: the fewest rounds of items
+// over the resident CTAs (two per SM up to three objectives, else one), an
+// item costing its row blocks and what it takes to stage and to flush a column
+// block: about 25 of them, 45 where one CTA does that alone. (100,000 points of
+// three objectives: 789 us with 1024 row blocks per item, 673 with 128; 60,000
+// of five: 490 with 128, 567 with 64, 639 with 1024.)
+int caller_chunk(int64_t n2, int m, int sms)
+{
+    const int64_t nrb = cdiv(n2, kTileRows), resident = (m <= 3 ? 2 : 1) * (int64_t)sms;
+    int best = kDomRowChunk;
+    int64_t least = INT64_MAX;
+    for (int c = kDomRowChunk; c >= kDomChunkMin; c >>= 1) {
+        const int64_t rounds = cdiv(cdiv(n2, kColBlock) * cdiv(nrb, c), resident);
+        const int64_t cost = rounds * (std::min<int64_t>(c, nrb) + (m <= 3 ? 25 : 45));
+        if (cost < least) {
+            least = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 Shape shape_for(int dev, int sms, int m, int64_t n2)
 {
     static std::once_flag env_once;  // shapes tuned by earlier processes
@@ -350,7 +372,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     if (cudaGetDevice(&dev) != cudaSuccess) return EMO_ERR_CUDA;
     for (auto& in : ins) {
         const Shape sh = shape_for(dev, di.sms, in.m, in.n2);
-        in.dom_chunk = sh.dom_chunk;
+        in.dom_chunk = in.mode == MODE_DOM ? caller_chunk(in.n2, in.m, di.sms) : sh.dom_chunk;
         in.cap_wide = sh.cap_wide;
         in.cap_narrow = sh.cap_narrow;
         in.ws_off = (uint64_t)off;
@@ -1088,7 +1110,7 @@ int32_t emo_device_report(char* buf, int32_t len)
                     {"k_stats", (const void*)k_stats, 0}, {"k_csr", (const void*)k_csr, 0},
                     {"k_niche", (const void*)k_niche, 0}, {"k_niche_oneshot", (const void*)k_niche_oneshot, 0},
                     {"k_peel_wave", (const void*)k_peel_wave, kPeelWaveDynSmem},
-                    {"k_hype", (const void*)k_hype, 0}, {"k_hype_counts", (const void*)k_hype_counts, hype_counts_smem(4)},
+                    {"k_hype", (const void*)k_hype, 0}, {"k_hype_counts", (const void*)k_hype_counts, hype_counts_smem(kSegKeys + 1)},
                     {"k_finish", (const void*)k_finish, 0}};
     for (const K& k : ks) {
         cudaFuncAttributes fa{};

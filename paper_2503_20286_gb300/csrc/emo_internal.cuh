@@ -263,44 +263,37 @@ __host__ __device__ __forceinline__ int64_t tile_index(int64_t rb, int64_t cb, i
     return tiles_before(rb, ncb) + (cb - rb / 32);
 }
 
-// Column-block prefix sets of the dominance kernel. Each 1024-column block
-// is split into two halves of 512 columns. For each key objective k
-// (objectives 2..m) the block stores:
+// Column-block prefix sets of the dominance kernels. The columns q of a
+// 1024-column block with f_k(q) >= x are a prefix of the block in the order of
+// f_k descending; the sets are stored so that each part of the block looks its
+// own prefix up. Per key objective k:
 //   fv   -- the block's 1024 values of f_k sorted descending (entry i at
 //           slot i ^ ((i / 32) % 32), which spreads a binary search's
 //           candidates over the shared-memory banks);
-//   cum0 -- cum0[j] = how many of the first j entries of fv lie in half 0
-//           (so a count j of values >= x splits into cum0[j] and j - cum0[j]);
-//   pb   -- for each half, the bitsets of its first c * cps columns in the
-//           order of f_k descending, c = 0..512/cps. Row c holds 32 words,
-//           words 0-15 from half 0 and 16-31 from half 1, so the word w of a
-//           tile row always comes from half w / 16;
-//   ord  -- (cps > 1 only) each half's local column indices in that order.
-//   per objective: float fv[1024] | uint16 cum0[1025] (+pad) | uint32 pb[512/cps + 1][32] | uint16 ord[2][512]
+//   cum  -- how many of the first j entries of fv lie in each part of the
+//           block, j = 0..1024;
+//   pb   -- row c holds, for every part, the bitset of its first c columns in
+//           that order (word w of a row is word w of a tile row);
+//   ord  -- (halves only) each half's local column indices in that order.
+// Up to kSegKeys keys: eight segments of 128 columns, every prefix stored:
+//   float fv[1024] | uint8 cum[1025][8] (+pad) | uint32 pb[129][32]
+// More keys (the segments' rows would not fit in shared memory): two halves of
+// 512 columns, every cps-th prefix stored, the rest completed from ord:
+//   float fv[1024] | uint16 cum0[1025] (+pad) | uint32 pb[512/cps + 1][32] | uint16 ord[2][512]
+constexpr int kSegKeys = 7;
+constexpr int kSegCols = 128, kSegs = kColBlock / kSegCols;
 constexpr int kPrefCumOff = kColBlock * 4;
+constexpr int kSegPbOff = kPrefCumOff + 8320;   // 1025 x 8 bytes rounded up to 128
 constexpr int kPrefPbOff = kPrefCumOff + 2176;  // 1025 uint16 rounded up to 128 bytes
-__host__ __device__ constexpr int colprep_log_cps(int K)
-{
-    return K <= 3 ? 0 : (K <= 5 ? 1 : (K <= 6 ? 2 : (K <= 9 ? 3 : 4)));
-}
+constexpr int kSegObjBytes = kSegPbOff + (kSegCols + 1) * 128;
+__host__ __device__ constexpr int colprep_log_cps(int K) { return K <= 9 ? 3 : 4; }
 __host__ __device__ constexpr int64_t colprep_ord_off(int K)
 {
     return kPrefPbOff + (((kColBlock / 2) >> colprep_log_cps(K)) + 1) * 32 * 4;
 }
-// Objectives with at most two prefix-set keys also carry a bucket index of
-// the block's descending values (header: lowest finite value, bucket scale;
-// then per bucket the first and one-past-last positions of the values in
-// it), which turns the search for a row's count into one lookup and a search
-// among the few values of one bucket.
-constexpr int kPrefBuckets = 4096;
-__host__ __device__ constexpr bool colprep_has_buckets(int K) { return K <= 2; }
-__host__ __device__ constexpr int64_t colprep_bkt_off(int K)
-{
-    return colprep_ord_off(K) + (colprep_log_cps(K) > 0 ? kColBlock * 2 : 0);
-}
 __host__ __device__ constexpr int64_t colprep_obj_bytes(int K)
 {
-    return colprep_bkt_off(K) + (colprep_has_buckets(K) ? 128 + kPrefBuckets * 4 : 0);
+    return K <= kSegKeys ? (int64_t)kSegObjBytes : colprep_ord_off(K) + kColBlock * 2;
 }
 
 // Bits per coordinate of a z-order grid over n items: about two cells per

@@ -4,16 +4,14 @@
 // Selection path (points in lexicographic order, so for p < q only "p
 // dominates q" is possible; it holds iff f_k(q) >= f_k(p) for every key
 // objective k = 2..m and the points are not identical):
-//   k_colprep -- for each 1024-column block, each half of 512 columns and
-//     each key objective k, sorts the half's columns by f_k (descending) and
-//     stores, every CPS sorted columns, the bitset of the columns seen so far.
-//     The set {q in half : f_k(q) >= f_k(p)} is then a prefix of that order:
-//     a checkpoint bitset plus at most CPS - 1 extra bits (CPS = 1 for m <= 4,
-//     so no extra bits at all).
-//   k_dom_pref<M> (m = 6; k_dom_pref_rt for m >= 7; up to five objectives are
-//     ranked without the matrix, k_fronts.cu) -- one warp per row
+//   k_colprep -- for each 1024-column block and each key objective k, the
+//     columns by f_k (descending): the set {q : f_k(q) >= f_k(p)} is then a
+//     prefix of that order. Up to seven keys every prefix of every 128-column
+//     segment is stored as a bitset.
+//   k_dom_pref<M> (m = 6..8; k_dom_pref_rt for m >= 9; up to five objectives
+//     are ranked without the matrix, k_fronts.cu) -- one warp per row
 //     block: each lane first counts, for its row and each objective, the
-//     columns of both halves that are >= (binary search). Then each half-warp
+//     columns of the block that are >= (binary search). Then each half-warp
 //     builds one row at a time (lanes 0-15 rows 0-15, lanes 16-31 rows 16-31),
 //     a lane owning 64 columns (two words): the words are the AND over the
 //     objectives of the prefix bitsets, masked by q > p (diagonal blocks) and
@@ -32,7 +30,8 @@ static_assert(kDomRowChunk / 16 * 16 < (1 << (4 + kDomNH)), "column counter over
 constexpr long long kCopyWaitCycles = 1ll << 32;
 constexpr int kHalf = kColBlock / 2;
 
-// Geometry of the per-objective prefix-set blocks (runtime form).
+// Geometry of the per-objective prefix-set blocks of halves (more than
+// kSegKeys keys).
 struct PrefGeom {
     int log_cps, cps, obj_bytes, ord_off;
     __device__ __forceinline__ explicit PrefGeom(int K)
@@ -40,14 +39,6 @@ struct PrefGeom {
           ord_off((int)colprep_ord_off(K))
     {
     }
-};
-
-template <int K>
-struct PrefShape {
-    static constexpr int LOG_CPS = colprep_log_cps(K);
-    static constexpr int CPS = 1 << LOG_CPS;
-    static constexpr int OBJ_BYTES = (int)colprep_obj_bytes(K);
-    static constexpr int ORD_OFF = (int)colprep_ord_off(K);
 };
 
 // Decode a dominance item of one problem: column blocks are served from the
@@ -90,15 +81,6 @@ __device__ __forceinline__ void flush_counts(VCount<NH>& vlo, VCount<NH>& vhi, i
     vhi = VCount<NH>();
 }
 
-// Bucket of x for a block's header (lowest finite value vmin, scale > 0 or
-// 0): non-decreasing in x, the same arithmetic where the index is built and
-// where it is searched.
-__device__ __forceinline__ int pref_bucket(float x, float vmin, float scale)
-{
-    const int b = __float2int_rz(__fmul_rn(__fsub_rn(x, vmin), scale));
-    return min(max(b, 0), kPrefBuckets - 1);
-}
-
 // ------------------------------------------------------------ k_colprep
 // Slot of entry i of a block's descending values (bank-spreading swizzle).
 __device__ __forceinline__ int fv_slot(int i) { return i ^ ((i >> 5) & 31); }
@@ -118,6 +100,57 @@ __device__ __forceinline__ int count_before512(const float* v, float x)
     return pos;
 }
 
+// Prefix sets of the eight 128-column segments from the block's descending
+// order (values s_v, columns s_i): warp w marks where segment w's columns fall
+// in the order, which gives both its share of every prefix (cum) and its own
+// order; then each word of a segment's bitsets is an OR over the columns
+// before, eight lanes (16 columns each) to a word.
+__device__ __forceinline__ void segment_sets(unsigned char* blk, const float* s_v, const uint16_t* s_i,
+                                             uint8_t* s_ord)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* fv = reinterpret_cast<float*>(blk);
+    uint8_t* cum = blk + kPrefCumOff;
+    uint32_t* pb = reinterpret_cast<uint32_t*>(blk + kSegPbOff);
+    for (int q = tid; q < kColBlock; q += blockDim.x) fv[fv_slot(q)] = s_v[q];
+    uint8_t* ord = s_ord + warp * kSegCols;  // columns within the segment
+    if (lane == 0) cum[warp] = 0;
+    int before = 0;
+    for (int q0 = 0; q0 < kColBlock; q0 += 32) {
+        const int col = s_i[q0 + lane];
+        const bool mine = col / kSegCols == warp;
+        const unsigned ballot = __ballot_sync(0xffffffffu, mine);
+        const int upto = before + __popc(ballot & ((2u << lane) - 1u));  // (lane 31: the mask wraps to all)
+        cum[(q0 + lane + 1) * kSegs + warp] = (uint8_t)upto;
+        if (mine) ord[upto - 1] = (uint8_t)(col % kSegCols);
+        before += __popc(ballot);
+    }
+    __syncwarp();
+    const int w = lane & 3, part = lane >> 2;
+    uint32_t own = 0u;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int col = ord[part * 16 + e];
+        own |= (col >> 5) == w ? 1u << (col & 31) : 0u;
+    }
+    uint32_t acc = own;
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, acc, o);
+        if (lane >= o) acc |= x;
+    }
+    acc = __shfl_up_sync(0xffffffffu, acc, 4);  // the parts before
+    if (part == 0) acc = 0u;
+    uint32_t* row = pb + warp * 4 + w;
+    if (part == 0) row[0] = 0u;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int col = ord[part * 16 + e];
+        acc |= (col >> 5) == w ? 1u << (col & 31) : 0u;
+        row[(part * 16 + e + 1) * 32] = acc;
+    }
+}
+
 __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int plast)
 {
     __shared__ float s_v[kColBlock];
@@ -125,9 +158,6 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
     __shared__ uint8_t s_mark[kColBlock];
     __shared__ uint32_t s_part[8][32];
     __shared__ int s_warp[32];
-    __shared__ float s_full[kColBlock];  // the full descending order (bucket index)
-    __shared__ float s_hdr[2];
-    __shared__ int s_bh[kPrefBuckets];  // bucket histogram
     __shared__ long long s_first[kMaxBatch + 1];  // items (column block, objective) before each problem
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // key objectives 2..m of the lexicographic order, or every objective of
@@ -163,15 +193,16 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
             s_i[q] = (uint16_t)q;
         }
         __syncthreads();
-        // bitonic sort: half ascending, then value descending, then local
-        // index ascending (positions 0..511 = half 0, 512..1023 = half 1)
+        // bitonic sort: value descending, then local index ascending; by halves
+        // each half by itself (positions 0..511 = half 0, 512..1023 = half 1)
+        const bool segs = K <= kSegKeys;
         for (int size = 2; size <= kColBlock; size <<= 1) {
             for (int stride = size >> 1; stride > 0; stride >>= 1) {
                 for (int t = tid; t < kColBlock / 2; t += blockDim.x) {
                     const int i = 2 * t - (t & (stride - 1)), j = i + stride;
                     const float vi = s_v[i], vj = s_v[j];
                     const int ii = s_i[i], ij = s_i[j];
-                    const int hi_ = ii >= kHalf, hj = ij >= kHalf;
+                    const int hi_ = !segs && ii >= kHalf, hj = !segs && ij >= kHalf;
                     const bool j_first = hj < hi_ || (hj == hi_ && (vj > vi || (vj == vi && ij < ii)));
                     const bool up = (i & size) == 0;
                     if (up == j_first) {
@@ -182,13 +213,16 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
                 __syncthreads();
             }
         }
+        if (segs) {
+            segment_sets(blk, s_v, s_i, s_mark);
+            __syncthreads();
+            continue;
+        }
         float* fv = reinterpret_cast<float*>(blk);
         uint16_t* cum0 = reinterpret_cast<uint16_t*>(blk + kPrefCumOff);
         uint32_t* pb = reinterpret_cast<uint32_t*>(blk + kPrefPbOff);
-        if (G.log_cps > 0) {
-            uint16_t* so = reinterpret_cast<uint16_t*>(blk + G.ord_off);
-            for (int q = tid; q < kColBlock; q += blockDim.x) so[q] = s_i[q];
-        }
+        uint16_t* so = reinterpret_cast<uint16_t*>(blk + G.ord_off);
+        for (int q = tid; q < kColBlock; q += blockDim.x) so[q] = s_i[q];
         // merge of the halves into the full descending order (ties: half 0
         // first); mark the half-0 positions
         for (int q = tid; q < kColBlock; q += blockDim.x) {
@@ -197,50 +231,6 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
                              (q < kHalf ? count_before512<true>(s_v + kHalf, x) : count_before512<false>(s_v, x));
             fv[fv_slot(rank)] = x;
             s_mark[rank] = q < kHalf;
-            if (colprep_has_buckets(K)) s_full[rank] = x;
-        }
-        if (colprep_has_buckets(K)) {
-            // bucket index: header (vmin, scale), then per bucket b the
-            // positions [lo, hi) of the values whose bucket is b (the
-            // bucket is non-increasing along the descending order)
-            __syncthreads();
-            float* hdr = reinterpret_cast<float*>(blk + colprep_bkt_off(K));
-            uint32_t* tab = reinterpret_cast<uint32_t*>(blk + colprep_bkt_off(K) + 128);
-            if (tid == 0) {
-                int nf = kColBlock;  // finite entries (padding columns hold -inf)
-                while (nf > 1 && !(s_full[nf - 1] > -INFINITY)) --nf;
-                const float vmax = s_full[0], vmin = s_full[nf - 1];
-                float sc = vmax > vmin ? (float)kPrefBuckets / (vmax - vmin) : 0.0f;
-                if (!(sc < 1e30f)) sc = 0.0f;  // overflowed span or tiny span: one bucket
-                s_hdr[0] = vmin;
-                s_hdr[1] = sc;
-                hdr[0] = vmin;
-                hdr[1] = sc;
-            }
-            __syncthreads();
-            const float vmin = s_hdr[0], sc = s_hdr[1];
-            // histogram of the values' buckets, then per bucket b:
-            // lo = #{bucket > b}, hi = #{bucket >= b} (a block scan)
-            constexpr int PER = kPrefBuckets / 256;
-            for (int b = tid; b < kPrefBuckets; b += blockDim.x) s_bh[b] = 0;
-            __syncthreads();
-            for (int q = tid; q < kColBlock; q += blockDim.x) atomicAdd(&s_bh[pref_bucket(s_full[q], vmin, sc)], 1);
-            __syncthreads();
-            int h[PER], sum = 0;
-#pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                h[e] = s_bh[tid * PER + e];
-                sum += h[e];
-            }
-            int tot;
-            int below = block_exclusive_scan<256>(sum, s_warp, tot);  // #{bucket < tid * PER}
-#pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                const int hi = kColBlock - below;
-                below += h[e];
-                tab[tid * PER + e] = (uint32_t)(kColBlock - below) | ((uint32_t)hi << 16);
-            }
-            __syncthreads();  // s_warp is scanned again below
         }
         // interleaved prefix bitsets: lane w builds word w from the sorted
         // columns of half w / 16; warp v covers checkpoints (v*seg, (v+1)*seg]
@@ -283,21 +273,21 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
 // ------------------------------------------------------------ k_dom_pref
 template <int K>
 struct PrefSmem {
-    alignas(128) unsigned char obj[K * PrefShape<K>::OBJ_BYTES];
+    alignas(128) unsigned char obj[K * kSegObjBytes];
     alignas(128) int32_t rs[kColBlock];
     int32_t cnt[kColBlock];
+    alignas(8) unsigned char st[16][K * 128];  // each warp's staged segment counts
     uint64_t bar;
     long long item;
     int skip;
 };
 
-// Packed counts of the block's values >= x in both halves of one objective:
-// t0 | t1 << 16 (binary search over the full descending order, then the
-// half-0 share of that prefix). Entry i of the order is stored at fv_slot(i):
-// the candidates of one search level are i = c * step - 1 for step >= 32, all
-// with the same low five bits, and the XOR with i / 32 puts them in distinct
-// shared-memory banks.
-__device__ __forceinline__ int count_ge_halves(const unsigned char* ob, float x)
+// How many of the block's values of one objective are >= x (binary search
+// over the full descending order). Entry i of the order is stored at
+// fv_slot(i): the candidates of one search level are i = c * step - 1 for
+// step >= 32, all with the same low five bits, and the XOR with i / 32 puts
+// them in distinct shared-memory banks.
+__device__ __forceinline__ int count_ge(const unsigned char* ob, float x)
 {
     const float* fv = reinterpret_cast<const float*>(ob);
     int pos = 0;
@@ -305,102 +295,101 @@ __device__ __forceinline__ int count_ge_halves(const unsigned char* ob, float x)
     for (int step = kColBlock / 2; step > 0; step >>= 1)
         if (fv[fv_slot(pos + step - 1)] >= x) pos += step;
     if (fv[fv_slot(pos)] >= x) ++pos;
+    return pos;
+}
+
+// The count split by halves: t0 | t1 << 16.
+__device__ __forceinline__ int count_ge_halves(const unsigned char* ob, float x)
+{
+    const int pos = count_ge(ob, x);
     const int t0 = reinterpret_cast<const uint16_t*>(ob + kPrefCumOff)[pos];
     return t0 | ((pos - t0) << 16);
 }
 
-// count_ge_halves through the bucket index (objectives with at most two
-// keys): every value of a higher bucket is >= x, every value of a lower one
-// < x, so the count is the bucket's first position plus the values >= x
-// among the bucket's own (a short search, usually over one or none).
+// Segment counts of the rows g * 8 .. + 7 and 16 + g * 8 .. + 7 of a row block
+// into the warp's staging area (8 bytes per objective and row): the count t[k]
+// of the lane's row split over the segments.
 template <int K>
-__device__ __forceinline__ int count_ge_halves_k(const unsigned char* ob, float x)
+__device__ __forceinline__ void stage_counts(const unsigned char* obj, unsigned char* st, const int (&t)[K], int g, int lane)
 {
-    if constexpr (!colprep_has_buckets(K)) {
-        return count_ge_halves(ob, x);
-    } else {
-        const float* fv = reinterpret_cast<const float*>(ob);
-        const float* hdr = reinterpret_cast<const float*>(ob + colprep_bkt_off(K));
-        const uint32_t e =
-            reinterpret_cast<const uint32_t*>(ob + colprep_bkt_off(K) + 128)[pref_bucket(x, hdr[0], hdr[1])];
-        int lo = (int)(e & 0xffffu), hi = (int)(e >> 16);
-        while (lo < hi) {  // first position of the bucket with a value < x
-            const int mid = (lo + hi) >> 1;
-            if (fv[fv_slot(mid)] >= x) lo = mid + 1;
-            else hi = mid;
-        }
-        const int t0 = reinterpret_cast<const uint16_t*>(ob + kPrefCumOff)[lo];
-        return t0 | ((lo - t0) << 16);
-    }
-}
-
-// Two words (columns 64 l .. 64 l + 63, l = lane % 16) of an objective's
-// prefix set for a count t of the lane's half.
-template <int LOG_CPS, int ORD_OFF>
-__device__ __forceinline__ unsigned long long prefix_word(const unsigned char* ob, int t, int l)
-{
-    const int c = t >> LOG_CPS;
-    unsigned long long w = *reinterpret_cast<const unsigned long long*>(ob + kPrefPbOff + c * 128 + l * 8);
-    if (LOG_CPS > 0) {
-        constexpr int CPS = 1 << LOG_CPS;
-        const int rem = t & (CPS - 1);
-        const uint16_t* so = reinterpret_cast<const uint16_t*>(ob + ORD_OFF) + (l >> 3) * kHalf;
+    __syncwarp();  // the rows before are read
+    if (((lane >> 3) & 1) == g) {
+        const int row = (lane & 7) + (lane >> 4) * 8;
 #pragma unroll
-        for (int e = 0; e < CPS - 1; ++e) {
-            const int col = so[min((c << LOG_CPS) + e, kHalf - 1)];
-            const bool hit = (e < rem) & ((col >> 6) == l);
-            w |= hit ? (1ull << (col & 63)) : 0ull;
-        }
+        for (int k = 0; k < K; ++k)
+            *reinterpret_cast<unsigned long long*>(st + k * 128 + row * 8) =
+                *reinterpret_cast<const unsigned long long*>(obj + k * kSegObjBytes + kPrefCumOff + t[k] * kSegs);
     }
-    return w;
+    __syncwarp();
 }
 
-// Keep columns q > p of the lane's 64 (diagonal blocks), drop identical points.
-template <bool DIAG, bool DUP>
-__device__ __forceinline__ unsigned long long row_masks(unsigned long long word, int64_t prow, int64_t cbase,
-                                                        const int32_t* __restrict__ rs, int l)
+// Two words (columns 64 l .. 64 l + 63, l = lane % 16) of the AND of the
+// objectives' prefix sets for the staged row jj (of the lane's half-warp): the
+// segment's share of each prefix, then that row of its bitsets. The 16 lanes
+// read one 8-byte entry and then 16 different bank pairs. (A shuffle of the
+// row's count and a look-up of its share instead of the staged bytes: one more
+// dependent access per objective, 575 us instead of 543 at 100,000 points of
+// eight objectives.)
+template <int K>
+__device__ __forceinline__ unsigned long long row_words(const unsigned char* obj_l, const unsigned char* st_l, int jj)
 {
-    if (DIAG) {
-        const int64_t off = prow - (cbase + 64 * l);
-        const int sh = (int)(off < 0 ? 0 : (off > 62 ? 63 : off + 1));  // shift count in [0, 63]
-        word &= off >= 63 ? 0ull : (off >= 0 ? ~0ull << sh : ~0ull);
-    }
-    if (DUP && word) {
-#pragma unroll 4
-        for (int bb = 0; bb < 64; ++bb) {
-            const int b = (bb + l) & 63;
-            if ((int64_t)rs[64 * l + b] <= prow) word &= ~(1ull << b);
-        }
+    unsigned long long word = ~0ull;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int c = st_l[k * 128 + jj * 8];
+        word &= *reinterpret_cast<const unsigned long long*>(obj_l + k * kSegObjBytes + kSegPbOff + c * 128);
     }
     return word;
 }
 
-// The 32 rows of row block rb in column block cb; t[k] is the packed count
-// (half 0 | half 1 << 16) of objective k for the lane's row.
-// DIAG: the row block overlaps the column block (keep q > p only).
-// DUP: a run of identical points may reach into the column block.
-template <int K, bool DIAG, bool DUP>
-__device__ __forceinline__ void pref_rows(const unsigned char* __restrict__ obj, const int32_t* __restrict__ rs,
-                                          const int (&t)[K], int64_t rowbase, int64_t cbase, uint32_t* tile,
-                                          VCount<kDomNH>& vlo, VCount<kDomNH>& vhi, int lane)
+// First column of the block (0 .. 1024) that row p may dominate: past p itself
+// (diagonal blocks) and past the points identical to p, which follow it in the
+// order -- the columns whose run starts at p or before. nv: the block's points.
+template <bool DUP>
+__device__ __forceinline__ int first_column(const int32_t* rs, int64_t p, int64_t cbase, int nv)
 {
-    using S = PrefShape<K>;
+    int lo = (int)min((int64_t)kColBlock, max((int64_t)0, p + 1 - cbase));
+    if (DUP) {
+        int hi = nv;  // run starts ascend: the first one beyond p
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((int64_t)rs[mid] <= p) lo = mid + 1;
+            else hi = mid;
+        }
+    }
+    return lo;
+}
+
+// Keep the columns from `first` on of the lane's 64. (With the run starts tested
+// column by column in every row, the few blocks of rows beside the diagonal
+// left one SM busy while the others had finished: 543 us instead of 462 at
+// 100,000 points of eight objectives on a grid.)
+__device__ __forceinline__ unsigned long long keep_from(unsigned long long word, int first, int l)
+{
+    const int off = first - 64 * l;
+    return off >= 64 ? 0ull : (off > 0 ? word & (~0ull << off) : word);
+}
+
+// The 32 rows of row block rb in column block cb; t[k] is the count of
+// objective k for the lane's row.
+// EDGE: rows keep only the columns from `first` (of the lane's row) on.
+template <int K, bool EDGE>
+__device__ __forceinline__ void pref_rows(const unsigned char* __restrict__ obj, unsigned char* st,
+                                          const int (&t)[K], int first, uint32_t* tile, VCount<kDomNH>& vlo, VCount<kDomNH>& vhi, int lane)
+{
     const int l = lane & 15, h = lane >> 4;
-    const unsigned psel = (l >> 3) ? 0x4432u : 0x4410u;  // byte selector of the lane's half count
     unsigned long long* dst = reinterpret_cast<unsigned long long*>(tile + h * 16 * 32) + l;
+    const unsigned char* const obj_l = obj + l * 8;
+    const unsigned char* const st_l = st + h * 64 + (l >> 1);
 #pragma unroll 1
     for (int g = 0; g < 2; ++g) {
+        stage_counts<K>(obj, st, t, g, lane);
         uint32_t xl[8], xh[8];
 #pragma unroll
         for (int jj = 0; jj < 8; ++jj) {
             const int j = g * 8 + jj, i = j + 16 * h;
-            unsigned long long word = ~0ull;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const int tk = (int)__byte_perm((unsigned)__shfl_sync(0xffffffffu, t[k], i), 0u, psel);
-                word &= prefix_word<S::LOG_CPS, S::ORD_OFF>(obj + k * S::OBJ_BYTES, tk, l);
-            }
-            word = row_masks<DIAG, DUP>(word, rowbase + i, cbase, rs, l);
+            unsigned long long word = row_words<K>(obj_l, st_l, jj);
+            if (EDGE) word = keep_from(word, __shfl_sync(0xffffffffu, first, i), l);
             __stcs(dst + j * 16, word);
             xl[jj] = (uint32_t)word;
             xh[jj] = (uint32_t)(word >> 32);
@@ -471,7 +460,6 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
                                                      unsigned long long* counter)
 {
     constexpr int K = M - 1, NW = 16;
-    using S = PrefShape<K>;
     extern __shared__ __align__(128) unsigned char smraw[];
     PrefSmem<K>& sm = *reinterpret_cast<PrefSmem<K>*>(smraw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -491,7 +479,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
         const int rows = d.in.dom_chunk;
         dom_decode(item - plan->dom_item_start[p], d.ncb, d.nrb, rows, cb, chunk);
         bool fatal = false;
-        if (!dom_stage(d, cb, K, S::OBJ_BYTES, sm.obj, sm.rs, sm.cnt, &sm.bar, &sm.skip, parity, fatal)) {
+        if (!dom_stage(d, cb, K, kSegObjBytes, sm.obj, sm.rs, sm.cnt, &sm.bar, &sm.skip, parity, fatal)) {
             if (fatal) break;
             continue;
         }
@@ -500,6 +488,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
         const int rb_lo = chunk * rows, rb_hi = min(rbmax, rb_lo + rows);
         const int dupcut = d.minrs[cb];
         const int64_t cbase = (int64_t)cb * kColBlock;
+        const int nv = (int)min((int64_t)kColBlock, n2 - cbase);
         // in registers: the tile stores could alias the plan, which would
         // otherwise reload these after every row block
         uint32_t* const Dm = d.D;
@@ -518,7 +507,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
             const int64_t pl = (int64_t)rb * kTileRows + lane;
             int t[K];
 #pragma unroll
-            for (int k = 0; k < K; ++k) t[k] = pl < n2 ? count_ge_halves_k<K>(sm.obj + k * S::OBJ_BYTES, key[k]) : 0;
+            for (int k = 0; k < K; ++k) t[k] = pl < n2 ? count_ge(sm.obj + k * kSegObjBytes, key[k]) : 0;
             {
                 const int rbn = rb + NW;
                 const int64_t pn = (int64_t)rbn * kTileRows + lane;
@@ -527,11 +516,10 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
             }
             const bool diag = (int64_t)rb * kTileRows + 31 >= cbase;
             const bool dup = rb * kTileRows + 31 >= dupcut;
-            const int64_t rowbase = (int64_t)rb * kTileRows;
             uint32_t* tile = Dm + tile_index(rb, cb, ncb) * (int64_t)(kTileRows * kTileWords);
-            if (dup) pref_rows<K, true, true>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
-            else if (diag) pref_rows<K, true, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
-            else pref_rows<K, false, false>(sm.obj, sm.rs, t, rowbase, cbase, tile, vlo, vhi, lane);
+            if (dup) pref_rows<K, true>(sm.obj, sm.st[warp], t, first_column<true>(sm.rs, pl, cbase, nv), tile, vlo, vhi, lane);
+            else if (diag) pref_rows<K, true>(sm.obj, sm.st[warp], t, first_column<false>(sm.rs, pl, cbase, nv), tile, vlo, vhi, lane);
+            else pref_rows<K, false>(sm.obj, sm.st[warp], t, 0, tile, vlo, vhi, lane);
         }
         dom_flush_item(d, cbase, vlo, vhi, sm.cnt, lane);
     }
@@ -544,9 +532,9 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref(Plan* plan, long long item_
 // prefix sets, and p dominates q iff q is in that set and is not identical to
 // p (all equal: p itself and its exact duplicates, found as the runs of the
 // lexicographic sort). Items: (column block, chunk of row blocks) over the
-// whole square; a half-warp builds one 1024-column row segment at a time
-// (a lane owns 64 columns), written into row p of D; column counts as in
-// k_dom_pref. m <= 5 (the blocks' prefix data must fit in shared memory).
+// whole square; a warp builds one 1024-column row segment at a time (a lane
+// owns 32 columns), written into row p of D; column counts as in k_dom_pref.
+// m <= 5 (the blocks' prefix data must fit in shared memory).
 // Set-up of the caller-order matrix after the sort: the objectives in the
 // caller's order padded with -inf to whole column blocks (the prefix sets of
 // every objective are built on them), and each point's run of identical
@@ -573,34 +561,93 @@ __global__ void k_dom_keys(Plan* plan)
     }
 }
 
+// A row of D starts at any word (its stride is the caller's, by default
+// ceil(n2 / 32) words), so the segment of a row that a column block covers
+// shares its first and last 32-byte sectors with the blocks beside it. A lane
+// therefore owns one word and a warp stores 128 contiguous bytes of one row;
+// the items run along the rows, so that neighbouring blocks write at about the
+// same time, and the stores are kept in L2 like any other, where the shared
+// sectors meet. 100,000 points of three objectives (1.25 GB, a stride of 3125
+// words): 885 us with two words per lane stored one by one, 761 so, 816 with
+// stores that leave L2 first.
+// (up to three objectives two CTAs fit on an SM)
+constexpr int kCallerNH = 8;  // high count planes: up to 4095 rows per lane and item
+template <int K>
+struct CallerShape {
+    static constexpr int NT = K <= 3 ? 512 : 1024, NW = NT / 32;
+    static_assert((kDomRowChunk + NW - 1) / NW * 32 < (1 << (4 + kCallerNH)), "column counter overflow");
+};
 template <int K>
 struct CallerSmem {
-    alignas(128) unsigned char obj[K * PrefShape<K>::OBJ_BYTES];
+    alignas(128) unsigned char obj[K * kSegObjBytes];
     int32_t cnt[kColBlock];
+    alignas(8) unsigned char st[CallerShape<K>::NW][K * 256];  // each warp's segment counts: 8 bytes per objective and row
     uint64_t bar;
     long long item;
     int skip;
 };
 
-template <int K>
-__global__ void __launch_bounds__(512, 1) k_dom_caller(Plan* plan, long long nitems, unsigned long long* counter)
+// The 32 rows of one row block in one column block; the lane's word of the
+// first row goes to row0, w0 is its index within a row. PLAIN: none of the
+// checks below can apply.
+template <int K, bool PLAIN>
+__device__ __forceinline__ void caller_rows(const unsigned char* obj, const unsigned char* st, int64_t rowbase,
+                                            int64_t cbase, int64_t n2, uint32_t* row0, int64_t w0, int64_t ld,
+                                            const int32_t* idx, int dup_lo, int dup_hi, VCount<kCallerNH>& vc, int lane)
 {
-    constexpr int NW = 16;
-    using S = PrefShape<K>;
+    const unsigned char* const obj_l = obj + kSegPbOff + lane * 4;
+    const unsigned char* const st_l = st + (lane >> 2);
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+        uint32_t x[8];
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+            const int i = g * 8 + jj;
+            uint32_t word = ~0u;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int c = st_l[k * 256 + i * 8];
+                word &= *reinterpret_cast<const uint32_t*>(obj_l + k * kSegObjBytes + c * 128);
+            }
+            if (!PLAIN) {
+                // not identical to p: p itself, and its duplicates
+                const int64_t p = rowbase + i;
+                const int dlo = __shfl_sync(0xffffffffu, dup_lo, i), dhi = __shfl_sync(0xffffffffu, dup_hi, i);
+                if (dhi > dlo) {
+                    for (int r = dlo; r < dhi; ++r) {
+                        const int64_t off = (int64_t)__ldg(&idx[r]) - cbase - 32 * lane;
+                        if (off >= 0 && off < 32) word &= ~(1u << off);
+                    }
+                } else {
+                    const int64_t off = p - cbase - 32 * lane;
+                    if (off >= 0 && off < 32) word &= ~(1u << off);
+                }
+                if (p >= n2) word = 0u;
+                if (p < n2 && w0 < ld) row0[i * ld] = word;  // words past ld (a short last block) are not stored
+            } else {
+                row0[i * ld] = word;
+            }
+            x[jj] = word;
+        }
+        vc.add8_warp(x);
+    }
+}
+
+template <int K>
+__global__ void __launch_bounds__(CallerShape<K>::NT, K <= 3 ? 2 : 1) k_dom_caller(Plan* plan, long long nitems,
+                                                                                 unsigned long long* counter)
+{
+    constexpr int NW = CallerShape<K>::NW;
     extern __shared__ __align__(128) unsigned char smraw[];
     CallerSmem<K>& sm = *reinterpret_cast<CallerSmem<K>*>(smraw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int l = lane & 15, h = lane >> 4;
-    const unsigned psel = (l >> 3) ? 0x4432u : 0x4410u;  // byte selector of the lane's half count
     if (tid == 0) mbar_init(&sm.bar, 1);
     __syncthreads();
     uint32_t parity = 0;
     const ProbDev& d = plan->p[0];
     const int64_t n2 = d.in.n2, ld = d.in.dom_ld;
-    const int nrb = d.nrb;
+    const int nrb = d.nrb, ncb = d.ncb;
     const int rows = d.in.dom_chunk;
-    const long long per_cb = cdiv(nrb, rows);
-    const bool st64 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(d.in.dom_out) & 7) == 0);
     const int32_t* const idx = d.idx + (int64_t)ld_volatile(&d.sc->idx_buf) * d.n2p;
     const int32_t* const spos = d.spos;
     const float* const ck = d.ckeys;
@@ -610,12 +657,12 @@ __global__ void __launch_bounds__(512, 1) k_dom_caller(Plan* plan, long long nit
         __syncthreads();
         const long long item = sm.item;
         if (item >= nitems) break;
-        const int cb = (int)(item / per_cb), chunk = (int)(item % per_cb);
+        const int cb = (int)(item % ncb), chunk = (int)(item / ncb);
         if (tid == 0) {
             sm.skip = ld_volatile(&d.sc->status) != 0;
             if (!sm.skip) {
                 fence_proxy_async_smem();
-                bulk_load(sm.obj, d.colpre + (int64_t)cb * (K * S::OBJ_BYTES), (uint32_t)(K * S::OBJ_BYTES), &sm.bar);
+                bulk_load(sm.obj, d.colpre + (int64_t)cb * (K * kSegObjBytes), (uint32_t)(K * kSegObjBytes), &sm.bar);
             }
         }
         for (int i = tid; i < kColBlock; i += blockDim.x) sm.cnt[i] = 0;
@@ -629,91 +676,52 @@ __global__ void __launch_bounds__(512, 1) k_dom_caller(Plan* plan, long long nit
         parity ^= 1u;
         const int64_t cbase = (int64_t)cb * kColBlock;
         const int rb_lo = chunk * rows, rb_hi = min(nrb, rb_lo + rows);
-        VCount<kDomNH> vlo, vhi;
-        // keys and duplicate run of the lane's row in the warp's next row block (prefetched)
-        float key[K];
-        int nlo = -1, nhi = 0;
-        {
-            const int64_t pn = (int64_t)(rb_lo + warp) * kTileRows + lane;
-            const bool ok = rb_lo + warp < rb_hi && pn < n2;
-#pragma unroll
-            for (int k = 0; k < K; ++k) key[k] = ok ? __ldg(&ck[pn * K + k]) : 0.0f;
-            if (ok) {
-                nlo = __ldg(&spos[pn]);
-                nhi = __ldg(&spos[n2 + pn]);
-            }
-        }
+        VCount<kCallerNH> vc;
+        unsigned char* const st = sm.st[warp];
         for (int rb = rb_lo + warp; rb < rb_hi; rb += NW) {
-            const int64_t pl = (int64_t)rb * kTileRows + lane;  // the lane's row (search)
-            int t[K];
+            const int64_t rowbase = (int64_t)rb * kTileRows, pl = rowbase + lane;  // the lane's row (search)
+            __syncwarp();  // the counts before are read
 #pragma unroll
-            for (int k = 0; k < K; ++k) t[k] = pl < n2 ? count_ge_halves_k<K>(sm.obj + k * S::OBJ_BYTES, key[k]) : 0;
+            for (int k = 0; k < K; ++k) {
+                const unsigned char* const ob = sm.obj + k * kSegObjBytes;
+                const int pos = pl < n2 ? count_ge(ob, __ldg(&ck[pl * K + k])) : 0;
+                *reinterpret_cast<unsigned long long*>(st + k * 256 + lane * 8) =
+                    *reinterpret_cast<const unsigned long long*>(ob + kPrefCumOff + pos * kSegs);
+            }
             // duplicates of the lane's row: sorted positions [dup_lo, dup_hi) when it has any
-            const int dup_lo = nlo >= 0 ? nlo : 0, dup_hi = nlo >= 0 ? nhi : 0;
-            {
-                const int rbn = rb + NW;
-                const int64_t pn = (int64_t)rbn * kTileRows + lane;
-                const bool ok = rbn < rb_hi && pn < n2;
-#pragma unroll
-                for (int k = 0; k < K; ++k) key[k] = ok ? __ldg(&ck[pn * K + k]) : 0.0f;
-                nlo = ok ? __ldg(&spos[pn]) : -1;
-                nhi = ok ? __ldg(&spos[n2 + pn]) : 0;
-            }
-#pragma unroll 1
-            for (int g = 0; g < 2; ++g) {
-                uint32_t xl[8], xh[8];
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    const int j = g * 8 + jj, i = j + 16 * h;  // row of the block this half-warp builds
-                    const int64_t p = (int64_t)rb * kTileRows + i;
-                    unsigned long long word = ~0ull;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        const int tk = (int)__byte_perm((unsigned)__shfl_sync(0xffffffffu, t[k], i), 0u, psel);
-                        word &= prefix_word<S::LOG_CPS, S::ORD_OFF>(sm.obj + k * S::OBJ_BYTES, tk, l);
-                    }
-                    // not identical to p: p itself, and its duplicates
-                    const int dlo = __shfl_sync(0xffffffffu, dup_lo, i), dhi = __shfl_sync(0xffffffffu, dup_hi, i);
-                    if (dhi > dlo) {
-                        for (int r = dlo; r < dhi; ++r) {
-                            const int64_t off = (int64_t)__ldg(&idx[r]) - cbase - 64 * l;
-                            if (off >= 0 && off < 64) word &= ~(1ull << off);
-                        }
-                    } else {
-                        const int64_t off = p - cbase - 64 * l;
-                        if (off >= 0 && off < 64) word &= ~(1ull << off);
-                    }
-                    if (p >= n2) word = 0ull;
-                    if (p < n2) {  // words past ld (a short last block) are not stored
-                        const int64_t w0 = (int64_t)cb * 32 + 2 * l;
-                        uint32_t* dst = Dout + p * ld + w0;
-                        if (st64 && w0 + 1 < ld) {
-                            __stcs(reinterpret_cast<unsigned long long*>(dst), word);
-                        } else {
-                            if (w0 < ld) __stcs(dst, (uint32_t)word);
-                            if (w0 + 1 < ld) __stcs(dst + 1, (uint32_t)(word >> 32));
-                        }
-                    }
-                    xl[jj] = (uint32_t)word;
-                    xh[jj] = (uint32_t)(word >> 32);
-                }
-                vlo.add8_warp(xl);
-                vhi.add8_warp(xh);
-            }
+            const int dup_lo = pl < n2 ? __ldg(&spos[pl]) : -1, dup_hi = dup_lo >= 0 ? __ldg(&spos[n2 + pl]) : -1;
+            __syncwarp();
+            // (the usual block of rows: all there, none with a duplicate, none
+            // among the block's columns, whole words to store)
+            const bool plain = rowbase + kTileRows <= n2 && cb * 32 + 32 <= ld &&
+                               (rowbase + kTileRows <= cbase || rowbase >= cbase + kColBlock) &&
+                               !__any_sync(0xffffffffu, dup_hi > dup_lo);
+            const int64_t w0 = (int64_t)cb * 32 + lane;
+            uint32_t* const row0 = Dout + rowbase * ld + w0;
+            if (plain) caller_rows<K, true>(sm.obj, st, rowbase, cbase, n2, row0, w0, ld, idx, dup_lo, dup_hi, vc, lane);
+            else caller_rows<K, false>(sm.obj, st, rowbase, cbase, n2, row0, w0, ld, idx, dup_lo, dup_hi, vc, lane);
         }
         // column counts of the item: shared-memory reduction, one global atomic per column
-        flush_counts(vlo, vhi, sm.cnt, lane);
-        __syncthreads();
-        if (d.in.dom_count)
+        if (d.in.dom_count) {
+            const int top = vc.top_plane();
+            if (top >= 0) {
+#pragma unroll 4
+                for (int b = 0; b < 32; ++b) {
+                    const int c = vc.count_upto(b, top);
+                    if (c) atomicAdd(&sm.cnt[b * 32 + lane], c);
+                }
+            }
+            __syncthreads();
             for (int q = tid; q < kColBlock; q += blockDim.x) {
                 const int c = sm.cnt[(q & 31) * 32 + (q >> 5)];
                 if (c && cbase + q < n2) atomicAdd(&d.in.dom_count[cbase + q], c);
             }
+        }
         __syncthreads();
     }
 }
 
-// Runtime-K variant for m >= 7 (compact code: loops over the key objectives
+// Runtime-K variant for m >= 9, prefix sets by halves (compact code: loops over the key objectives
 // are not unrolled; the packed half counts of a row block are staged in
 // shared memory).
 __global__ void __launch_bounds__(512, 1) k_dom_pref_rt(Plan* plan, long long item_lo, long long item_hi,
@@ -758,6 +766,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref_rt(Plan* plan, long long it
         const int rb_lo = chunk * rows, rb_hi = min(rbmax, rb_lo + rows);
         const int dupcut = d.minrs[cb];
         const int64_t cbase = (int64_t)cb * kColBlock;
+        const int nv = (int)min((int64_t)kColBlock, n2 - cbase);
         uint32_t* const Dm = d.D;
         const float* const keys = d.keys;
         const int ncb = d.ncb;
@@ -769,6 +778,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref_rt(Plan* plan, long long it
             __syncwarp();
             const bool diag = (int64_t)rb * kTileRows + 31 >= cbase;
             const bool dup = rb * kTileRows + 31 >= dupcut;
+            const int first = dup ? first_column<true>(rs, pl, cbase, nv) : (diag ? first_column<false>(rs, pl, cbase, nv) : 0);
             uint32_t* tile = Dm + tile_index(rb, cb, ncb) * (int64_t)(kTileRows * kTileWords);
             unsigned long long* dst = reinterpret_cast<unsigned long long*>(tile + h * 16 * 32) + l;
 #pragma unroll 1
@@ -794,9 +804,7 @@ __global__ void __launch_bounds__(512, 1) k_dom_pref_rt(Plan* plan, long long it
                         }
                         word &= wk;
                     }
-                    const int64_t prow = (int64_t)rb * kTileRows + i;
-                    if (dup) word = row_masks<true, true>(word, prow, cbase, rs, l);
-                    else if (diag) word = row_masks<true, false>(word, prow, cbase, rs, l);
+                    if (diag | dup) word = keep_from(word, __shfl_sync(0xffffffffu, first, i), l);
                     __stcs(dst + j * 16, word);
                     xl[jj] = (uint32_t)word;
                     xh[jj] = (uint32_t)(word >> 32);
@@ -975,12 +983,12 @@ static cudaError_t launch_caller_k(Plan* plan, int sms, cudaStream_t s, long lon
     cudaError_t e = cudaFuncSetAttribute(k_dom_caller<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dom_caller<K>, 512, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dom_caller<K>, CallerShape<K>::NT, smem);
     if (e != cudaSuccess) return e;
     long long grid = (long long)sms * (occ > 0 ? occ : 1);
     if (grid > nitems) grid = nitems;
     if (grid < 1) return cudaSuccess;
-    k_dom_caller<K><<<(unsigned)grid, 512, smem, s>>>(plan, nitems, counter);
+    k_dom_caller<K><<<(unsigned)grid, CallerShape<K>::NT, smem, s>>>(plan, nitems, counter);
     return cudaGetLastError();
 }
 
@@ -1018,6 +1026,8 @@ cudaError_t launch_dominance_tri_range(int m, Plan* plan, int sms, cudaStream_t 
     (void)plast;
     switch (m) {
     case 6: return launch_tri_m<6>(plan, sms, s, lo, hi, counter);
+    case 7: return launch_tri_m<7>(plan, sms, s, lo, hi, counter);
+    case 8: return launch_tri_m<8>(plan, sms, s, lo, hi, counter);
     default:
         if (m <= kTreeMaxM || m > kMaxM) return cudaErrorInvalidValue;  // (fewer objectives need no matrix)
         return launch_tri_rt(m - 1, plan, sms, s, lo, hi, counter);

@@ -279,19 +279,40 @@ __device__ __forceinline__ void hype_contributions(const Plan* plan, const Group
     for (int64_t t = t0; t < want; t += stride) d.flag[__ldcg(&sorted[t])] = 1;
 }
 
+// Word w of the set of an objective's first pos columns in the block's
+// descending order, from the sets by segments and by halves.
+__device__ __forceinline__ uint32_t segment_word(const unsigned char* ob, int pos, int w)
+{
+    const int c = ob[kPrefCumOff + pos * kSegs + (w >> 2)];
+    return reinterpret_cast<const uint32_t*>(ob + kSegPbOff)[c * 32 + w];
+}
+__device__ __forceinline__ uint32_t halves_word(const unsigned char* ob, int K, int pos, int w)
+{
+    const int half = w >> 4, log_cps = colprep_log_cps(K);
+    const int h0 = reinterpret_cast<const uint16_t*>(ob + kPrefCumOff)[pos];
+    const int th = half ? pos - h0 : h0, c = th >> log_cps;
+    uint32_t pre = reinterpret_cast<const uint32_t*>(ob + kPrefPbOff)[c * 32 + w];
+    const uint16_t* ord = reinterpret_cast<const uint16_t*>(ob + colprep_ord_off(K)) + half * (kColBlock / 2);
+    for (int e = c << log_cps; e < th; ++e) {
+        const int col = ord[e];  // block-local
+        if ((col >> 5) == w) pre |= 1u << (col & 31);
+    }
+    return pre;
+}
+
 // (C) The dominator count c_i of every sample, from the column-block prefix
 // sets that the dominance stage built (points in lexicographic order). In
 // column block cb the points with f_1 <= s_1 are its first t1 positions (f_1
 // ascends along the order); for each key objective k >= 2 the points with
 // f_k <= s_k are the complement of the block's prefix of f_k-descending
-// order that holds the values > s_k (one prefix bitset per half of 512
-// columns, plus at most cps - 1 single bits). So
+// order that holds the values > s_k (its share of each part of the block, see
+// emo_internal.cuh). So
 //   c_i = sum over blocks of popc(first-t1 mask AND complemented prefix sets),
 // the count of every point with F_p <= S_i in all objectives. Items are
 // (column block, range of samples): the CTA copies the block's prefix data
 // (all key objectives, contiguous) into shared memory with one bulk copy and
 // gathers the block's f_1 values; each warp then takes 32 samples at a time:
-// lane = sample for the binary searches (t1 and the packed half counts), then
+// lane = sample for the binary searches (t1 and the counts), then
 // lane = word of the block for each of the 32 samples (AND, popcount, warp
 // sum), and one atomic add per sample and item.
 // The samples [s_lo, s_hi) against the staged column block (see
@@ -299,12 +320,11 @@ __device__ __forceinline__ void hype_contributions(const Plan* plan, const Group
 // then sized for the largest m and the loops run to the problem's m).
 template <int MM>
 __device__ __forceinline__ void hype_count_block(const ProbDev& d, const unsigned char* smraw, const float* s_f1,
-                                                 int64_t s_lo, int64_t s_hi, int nvalid, int64_t obj_bytes,
-                                                 int64_t ord_off, int log_cps)
+                                                 int64_t s_lo, int64_t s_hi, int nvalid)
 {
     const int m = MM == kMaxM ? d.in.m : MM, K = m - 1;
+    const int obj_bytes = (int)colprep_obj_bytes(K);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int half = lane >> 4;
     for (int64_t s0 = s_lo + (int64_t)warp * 32; s0 < s_hi; s0 += (int64_t)nw * 32) {
         const int64_t si = s0 + lane;
         const bool live = si < s_hi;
@@ -312,7 +332,7 @@ __device__ __forceinline__ void hype_count_block(const ProbDev& d, const unsigne
 #pragma unroll
         for (int k = 0; k < MM; ++k) sv[k] = (live && k < m) ? __ldcg(&d.rhat[si * m + k]) : -INFINITY;
         // lane = sample: positions with f_1 <= s_1, and per key objective the
-        // counts of values > s_k in each half (packed t0 | t1 << 16)
+        // count of values > s_k
         int t1;
         {
             int pos = 0;
@@ -323,12 +343,12 @@ __device__ __forceinline__ void hype_count_block(const ProbDev& d, const unsigne
             t1 = live ? min(pos, nvalid) : 0;
         }
         if (!__any_sync(0xffffffffu, t1 > 0)) continue;
-        int packed[MM - 1];
+        int above[MM - 1];
 #pragma unroll
         for (int k = 0; k < MM - 1; ++k) {
-            packed[k] = 0;
+            above[k] = 0;
             if (k < K) {
-                const unsigned char* ob = smraw + (int64_t)k * obj_bytes;
+                const unsigned char* ob = smraw + k * obj_bytes;
                 const float* fv = reinterpret_cast<const float*>(ob);
                 const float x = sv[k + 1];
                 int pos = 0;
@@ -336,8 +356,7 @@ __device__ __forceinline__ void hype_count_block(const ProbDev& d, const unsigne
                 for (int step = kColBlock / 2; step > 0; step >>= 1)
                     if (fv[hype_fv_slot(pos + step - 1)] > x) pos += step;
                 if (fv[hype_fv_slot(pos)] > x) ++pos;
-                const int h0 = reinterpret_cast<const uint16_t*>(ob + kPrefCumOff)[pos];
-                packed[k] = h0 | ((pos - h0) << 16);
+                above[k] = pos;
             }
         }
         // lane = word (block columns 32 lane .. 32 lane + 31)
@@ -349,19 +368,10 @@ __device__ __forceinline__ void hype_count_block(const ProbDev& d, const unsigne
 #pragma unroll
             for (int k = 0; k < MM - 1; ++k) {  // every lane: the loop holds warp shuffles
                 if (k < K) {
-                    const int pk = __shfl_sync(0xffffffffu, packed[k], j);
-                    const int th = half ? (pk >> 16) : (pk & 0xffff);
-                    const unsigned char* ob = smraw + (int64_t)k * obj_bytes;
-                    const int c = th >> log_cps;
-                    uint32_t pre = reinterpret_cast<const uint32_t*>(ob + kPrefPbOff)[c * 32 + lane];
-                    if (log_cps > 0) {
-                        const uint16_t* ord = reinterpret_cast<const uint16_t*>(ob + ord_off) + half * (kColBlock / 2);
-                        for (int e = c << log_cps; e < th; ++e) {
-                            const int col = ord[e];
-                            if ((col >> 5) == lane) pre |= 1u << (col & 31);  // col: block-local
-                        }
-                    }
-                    w &= ~pre;
+                    const int pos = __shfl_sync(0xffffffffu, above[k], j);
+                    const unsigned char* ob = smraw + k * obj_bytes;
+                    w &= ~(MM - 1 <= kSegKeys || K <= kSegKeys ? segment_word(ob, pos, lane)
+                                                               : halves_word(ob, K, pos, lane));
                 }
             }
             const int tot = __reduce_add_sync(0xffffffffu, __popc(w));
@@ -386,10 +396,8 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_hype_counts(Plan* plan)
         if (in.mode != MODE_HYPE) continue;
         const int m = in.m, K = m - 1, ns = in.n_r, ncb = d.ncb;
         const int64_t n2 = in.n2;
-        const int log_cps = colprep_log_cps(K);
-        const int64_t obj_bytes = colprep_obj_bytes(K), ord_off = colprep_ord_off(K);
-        const uint32_t blk_bytes = (uint32_t)(K * obj_bytes);
-        float* s_f1 = reinterpret_cast<float*>(smraw + align_up(blk_bytes, 128));
+        const uint32_t blk_bytes = (uint32_t)(K * colprep_obj_bytes(K));
+        float* s_f1 = reinterpret_cast<float*>(smraw + blk_bytes);
         const int32_t* idx = d.idx + (int64_t)ld_volatile(&d.sc->idx_buf) * d.n2p;
         const int64_t nsr = max((int64_t)1, min(cdiv(ns, 32), cdiv(2 * (int64_t)gridDim.x, ncb)));
         for (int64_t item = blockIdx.x; item < (int64_t)ncb * nsr; item += gridDim.x) {
@@ -418,10 +426,10 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_hype_counts(Plan* plan)
             }
             parity ^= 1u;
             switch (m) {  // compile-time objective counts keep the per-sample state in registers
-            case 2: hype_count_block<2>(d, smraw, s_f1, s_lo, s_hi, nvalid, obj_bytes, ord_off, log_cps); break;
-            case 3: hype_count_block<3>(d, smraw, s_f1, s_lo, s_hi, nvalid, obj_bytes, ord_off, log_cps); break;
-            case 4: hype_count_block<4>(d, smraw, s_f1, s_lo, s_hi, nvalid, obj_bytes, ord_off, log_cps); break;
-            default: hype_count_block<kMaxM>(d, smraw, s_f1, s_lo, s_hi, nvalid, obj_bytes, ord_off, log_cps);
+            case 2: hype_count_block<2>(d, smraw, s_f1, s_lo, s_hi, nvalid); break;
+            case 3: hype_count_block<3>(d, smraw, s_f1, s_lo, s_hi, nvalid); break;
+            case 4: hype_count_block<4>(d, smraw, s_f1, s_lo, s_hi, nvalid); break;
+            default: hype_count_block<kMaxM>(d, smraw, s_f1, s_lo, s_hi, nvalid);
             }
         }
     }
@@ -431,7 +439,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_hype_counts(Plan* plan)
 int hype_counts_smem(int m)
 {
     const int K = m - 1;
-    return (int)(align_up(K * colprep_obj_bytes(K), 128) + kColBlock * 4);
+    return (int)(K * colprep_obj_bytes(K)) + kColBlock * 4;
 }
 
 }  // namespace emo
