@@ -16,9 +16,16 @@ struct RadixSmem {
     int hist[kRadix];
     int off[kRadix];
     int wc[kCoopThreads / 32][kRadix];
-    int tot[kRadix];
+    int tot[kRadix / 32];
     int skip;
 };
+
+// CTAs that a pass over n items is spread over.
+constexpr int kRadixItems = 2048;  // items per CTA
+__device__ __forceinline__ int radix_ctas(const Group& g, int64_t n)
+{
+    return (int)max((int64_t)1, min((int64_t)g.size, cdiv(n, kRadixItems)));
+}
 
 template <typename KeyFn>
 __device__ bool radix_pass(const ProbDev& d, const Group& g, int gs, long long budget, int64_t n,
@@ -29,6 +36,7 @@ __device__ bool radix_pass(const ProbDev& d, const Group& g, int gs, long long b
     int (*s_wc)[kRadix] = rsm.wc;
     int* s_tot = rsm.tot;
     int& s_skip = rsm.skip;
+    static_assert(kCoopThreads == 2 * kRadix, "thread layout");
     const int tid = threadIdx.x, warp = tid >> 5;
     const bool active = g.rank < gs;
     const int64_t chunk = cdiv(n, gs);
@@ -44,28 +52,45 @@ __device__ bool radix_pass(const ProbDev& d, const Group& g, int gs, long long b
     if (!group_sync(g, d.sc, budget)) return false;
 
     // digit offsets of this CTA: all earlier digits + same digit of earlier CTAs
+    // (two threads per digit, each over half of the CTAs, then a scan by warps:
+    // with one thread adding up the 256 totals a pass over 100,000 points took
+    // 8 us longer)
     if (tid == 0) s_skip = 0;
-    __syncthreads();
-    for (int dg = tid; dg < kRadix; dg += blockDim.x) {
+    {
+        const int dg = tid & (kRadix - 1), half = tid >> kRadixBits, mid = (gs + 1) / 2;
+        const int end = half ? gs : mid;
         int col = 0, pre = 0;
-        for (int c = 0; c < gs; ++c) {
-            int v = __ldcg(&d.hist[c * kRadix + dg]);
+#pragma unroll 8
+        for (int c = half ? mid : 0; c < end; ++c) {
+            const int v = __ldcg(&d.hist[c * kRadix + dg]);
             col += v;
             if (c < g.rank) pre += v;
         }
-        s_tot[dg] = col;
-        s_off[dg] = pre;
-        if ((int64_t)col == n) s_skip = 1;
+        s_wc[half][dg] = col;
+        s_wc[2 + half][dg] = pre;
     }
     __syncthreads();
-    if (tid == 0) {
-        int run = 0;
-        for (int dg = 0; dg < kRadix; ++dg) { int c = s_tot[dg]; s_tot[dg] = run; run += c; }
+    int col = 0, incl = 0;
+    if (tid < kRadix) {
+        col = s_wc[0][tid] + s_wc[1][tid];
+        s_off[tid] = s_wc[2][tid] + s_wc[3][tid];
+        if ((int64_t)col == n) s_skip = 1;
+        incl = col;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((tid & 31) >= o) incl += x;
+        }
+        if ((tid & 31) == 31) s_tot[warp] = incl;
     }
     __syncthreads();
     skipped = s_skip != 0;
     if (!skipped) {
-        for (int dg = tid; dg < kRadix; dg += blockDim.x) s_off[dg] += s_tot[dg];
+        if (tid < kRadix) {
+            int before = incl - col;
+            for (int w = 0; w < warp; ++w) before += s_tot[w];
+            s_off[tid] += before;
+        }
         for (int i = tid; i < (kCoopThreads / 32) * kRadix; i += blockDim.x) (&s_wc[0][0])[i] = 0;
         __syncthreads();
         // stable scatter, one tile of blockDim elements at a time

@@ -262,7 +262,7 @@ __device__ __forceinline__ void hype_contributions(const Plan* plan, const Group
         for (int64_t t = t0; t < nL; t += stride) d.flag[__ldcg(&L[t])] = 1;
         return;
     }
-    const int gs = (int)max((int64_t)1, min((int64_t)g.size, cdiv(nL, 4096)));
+    const int gs = radix_ctas(g, nL);
     int buf = 0;
     for (int shift = 0; shift < 64; shift += kRadixBits) {
         const int32_t* src = d.llist + (int64_t)buf * n2;

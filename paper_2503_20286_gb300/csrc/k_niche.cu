@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_csr(Plan* plan)
     while ((1ll << bits) < (long long)nr) ++bits;
     int buf = 0;
     __shared__ RadixSmem rsm;
-    const int gs = (int)max((int64_t)1, min((int64_t)g.size, cdiv(nL, 4096)));
+    const int gs = radix_ctas(g, nL);
     for (int shift = 0; shift < bits; shift += kRadixBits) {
         const int32_t* src = d.llist + (int64_t)buf * n2;
         int32_t* dst = d.llist + (int64_t)(buf ^ 1) * n2;

@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
     if (ld_volatile(&d.sc->status) != 0) return;
     const int64_t n2 = in.n2;
     const int m = in.m;
-    const int gs = (int)max((int64_t)1, min((int64_t)g.size, cdiv(n2, 4096)));
+    const int gs = radix_ctas(g, n2);
     const float* F = in.F;
     __shared__ RadixSmem rsm;
     if (!lex_ordered(in)) return;  // ranks given, or ranked by the z-order tree
@@ -255,22 +255,49 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
     // by one thread. If some run is longer than kShortRun, the full stable
     // LSD sort over all objectives runs instead (from the index order).
     int buf = 0;
-    const uint32_t* kor = d.sc->kor;  // written by k_prep
-    const uint32_t* kinv = d.sc->kinv;
-    auto sort_by = [&](int k) -> bool {
-        const uint32_t varies = __ldcg(&kor[k]) & __ldcg(&kinv[k]);
-        for (int shift = 0; shift < 32; shift += kRadixBits) {
-            if (((varies >> shift) & (kRadix - 1)) == 0) continue;  // every point has the same digit
+    // A stable sort by the objectives [ka, kb) takes the bits between the lowest
+    // and the highest that vary over the points (k_prep), objective kb - 1
+    // lowest, as one string of digits: on a grid of 64 values eight objectives
+    // need 10 passes instead of 18 (100,000 points: 354 us, 517 by whole bytes).
+    __shared__ uint32_t s_lo[kMaxM], s_width[kMaxM];
+    __shared__ int s_at[kMaxM];
+    auto sort_by = [&](int ka, int kb) -> bool {
+        __syncthreads();
+        int bits = 0;
+        for (int k = kb - 1; k >= ka; --k) {
+            const uint32_t varies = __ldcg(&d.sc->kor[k]) & __ldcg(&d.sc->kinv[k]);
+            const int lo = varies ? __ffs(varies) - 1 : 0, width = varies ? 32 - __clz(varies) - lo : 0;
+            if (threadIdx.x == 0) {
+                s_lo[k] = lo;
+                s_width[k] = width;
+                s_at[k] = bits;
+            }
+            bits += width;
+        }
+        __syncthreads();
+        for (int at = 0; at < bits; at += kRadixBits) {
+            int k1 = kb - 1, k0 = ka;  // the objectives with bits in this digit
+            while (k1 > ka && s_at[k1] + (int)s_width[k1] <= at) --k1;
+            while (k0 < k1 && s_at[k0] >= at + kRadixBits) ++k0;
             const int32_t* src = d.idx + (int64_t)buf * d.n2p;
             int32_t* dst = d.idx + (int64_t)(buf ^ 1) * d.n2p;
             bool skipped = false;
-            auto key = [&](int32_t v) { return float_key(__ldg(&F[(int64_t)v * m + k])); };
-            if (!radix_pass(d, g, gs, budget, n2, src, dst, shift, key, skipped, rsm)) return false;
+            auto key = [&](int32_t v) {
+                uint32_t digit = 0u;
+                for (int k = k0; k <= k1; ++k) {
+                    const uint32_t w = s_width[k], x = float_key(__ldg(&F[(int64_t)v * m + k])) >> s_lo[k];
+                    const uint32_t val = w < 32 ? x & ((1u << w) - 1u) : x;
+                    const int rel = s_at[k] - at;
+                    digit |= rel >= 0 ? val << rel : val >> -rel;
+                }
+                return digit;
+            };
+            if (!radix_pass(d, g, gs, budget, n2, src, dst, 0, key, skipped, rsm)) return false;
             if (!skipped) buf ^= 1;
         }
         return true;
     };
-    if (!sort_by(0)) return;
+    if (!sort_by(0, 1)) return;
     {
         constexpr int kShortRun = 32;
         int32_t* cur = d.idx + (int64_t)buf * d.n2p;
@@ -315,8 +342,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
             for (int64_t s = (int64_t)g.rank * blockDim.x + threadIdx.x; s < n2; s += stride) id[s] = (int32_t)s;
             buf ^= 1;
             if (!group_sync(g, d.sc, budget)) return;
-            for (int k = m - 1; k >= 0; --k)
-                if (!sort_by(k)) return;
+            if (!sort_by(0, m)) return;
         }
     }
     if (g.rank == 0 && threadIdx.x == 0) d.sc->idx_buf = buf;
@@ -356,14 +382,13 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_sort(Plan* plan)
         d.hist[g.rank] = mx;
     }
     if (!group_sync(g, d.sc, budget)) return;
-    __shared__ int s_carry;
-    if (threadIdx.x == 0) {
-        int c = 0;
-        for (int r = 0; r < g.rank; ++r) c = max(c, __ldcg(&d.hist[r]));
-        s_carry = c;
-    }
+    int carry = 0;  // the last run start before this CTA's share
+    for (int r = threadIdx.x; r < g.rank; r += blockDim.x) carry = max(carry, __ldcg(&d.hist[r]));
+    carry = __reduce_max_sync(0xffffffffu, carry);
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = carry;
     __syncthreads();
-    int carry = s_carry;
+    for (int w = 0; w < kCoopThreads / 32; ++w) carry = max(carry, s_warp[w]);
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t base = lo; base < hi; base += blockDim.x) {
         const int64_t s = base + threadIdx.x;
