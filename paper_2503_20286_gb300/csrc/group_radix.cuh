@@ -21,7 +21,8 @@ struct RadixSmem {
 };
 
 // CTAs that a pass over n items is spread over.
-constexpr int kRadixItems = 2048;  // items per CTA
+// (100,000 points of eight objectives: 1,533 us with 2,048, 1,499 with 1,024)
+constexpr int kRadixItems = 1024;
 __device__ __forceinline__ int radix_ctas(const Group& g, int64_t n)
 {
     return (int)max((int64_t)1, min((int64_t)g.size, cdiv(n, kRadixItems)));
