@@ -40,7 +40,9 @@
 namespace emo {
 
 // ------------------------------------------------------------ k_fronts
-constexpr int kFrontRound = 128;       // leaves of a CTA looked at before their searches run
+// Leaves of a CTA looked at before their searches run (a round ends with its
+// longest search: 400,000 points, 82 leaves per CTA, 1.63 ms with 64, 1.44 with 128).
+constexpr int kFrontRound = 128;
 constexpr int kFrontQueue = kFrontRound * 32;  // searches of a round
 
 struct FrontSmem {

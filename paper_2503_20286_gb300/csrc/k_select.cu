@@ -392,11 +392,21 @@ __device__ __forceinline__ float assoc_chord(float c1, float nrm)
 }
 
 constexpr int kAssocWarps = 8;
-constexpr int kAssocFill = 2432;  // warps that keep the GPU busy: 16 per SM
+constexpr int kAssocFill = 2432;   // warps that keep the GPU busy: 16 per SM (up to five objectives 24 fit, 2% more)
+// Tasks are uneven (a warp whose points lie apart visits several times the
+// leaves of another), so up to kAssocShare lanes per point there are four for
+// each of those warps where the references fill more than one node; with more
+// lanes per point the search itself loses (10,056 points: 16 lanes each 18 us
+// longer), and a few leaves make tasks too short to split (156 references: 43 us,
+// 70 with more tasks). With one task per warp 22,170 points of five objectives
+// and 20,475 references kept the SMs active for half of 258 us; 247 -> 206 us,
+// 200,864 points of three objectives and 200,028 references 282 -> 223 us.
+constexpr int kAssocTasks = 9728;
+constexpr int kAssocShare = 8;
 constexpr int kAssocMany = 6;     // balls within the warp's reach from which each point is asked
 
 template <int M>
-__global__ void __launch_bounds__(kAssocWarps * 32) k_assoc(Plan* plan, int pfirst, int plast)
+__global__ void __launch_bounds__(kAssocWarps * 32, M <= kTreeMaxM ? 3 : 2) k_assoc(Plan* plan, int pfirst, int plast)
 {
     constexpr int MP = (M + 3) / 4 * 4, V = MP / 4;
     __shared__ float4 s_u[kAssocWarps][32 * V];
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(kAssocWarps * 32) k_assoc(Plan* plan, int pfir
     __shared__ int s_first[kMaxBatch + 1];
     __shared__ int s_share;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // lanes per point: enough warps for the GPU, at most a warp per point;
+    // lanes per point: enough tasks for the GPU, at most a warp per point;
     // tasks (warps' worth of points) before each problem
     if (tid == 0) {
         long long tot = 0;
@@ -412,9 +422,14 @@ __global__ void __launch_bounds__(kAssocWarps * 32) k_assoc(Plan* plan, int pfir
             const ProbDev& d = plan->p[p];
             return d.in.mode == MODE_SELECT && d.in.m == M && ld_volatile(&d.sc->status) == 0 ? ld_volatile(&d.sc->nS) : 0;
         };
-        for (int p = pfirst; p < plast; ++p) tot += count(p);
+        bool large = false;
+        for (int p = pfirst; p < plast; ++p) {
+            const int c = count(p);
+            tot += c;
+            large |= c > 0 && plan->p[p].nrnode > 1;
+        }
         int share = 1;
-        while (share < 32 && tot * share < (long long)kAssocFill * 32) share *= 2;
+        while (share < 32 && tot * share < 32ll * (large && share < kAssocShare ? kAssocTasks : kAssocFill)) share *= 2;
         int acc = 0;
         for (int p = pfirst; p < plast; ++p) {
             s_first[p - pfirst] = acc;
