@@ -31,8 +31,8 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
     // the grid in proportion to the work, at least one CTA for every problem that
     // the kind serves and at most the problem's cap. Wide groups by n2^2
     // (dominance tiles read per front), narrow ones by n2, tree groups by the CTA
-    // time to expect: 0.09 us per point of two or three objectives, 0.19 of
-    // five. A tree group gets the CTAs that hold its leaves in shared memory
+    // time to expect: 0.13 us per point of two objectives (many fronts), 0.09 of
+    // three, 0.19 of five. A tree group gets the CTAs that hold its leaves in shared memory
     // before the rest is shared out, where the grid suffices for that (38,524
     // points of two objectives: 18 us a front with the leaves in global memory,
     // 13 in shared). CTAs beyond the groups serve no problem.
@@ -45,7 +45,7 @@ __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
             const ProbIn& in = a.in[p];
             const float n = (float)in.n2;
             if (kind == GRP_WIDE) return tree_ranked(in) && in.mode != MODE_HYPE ? 0.0f : n * n;
-            if (kind == GRP_TREE) return tree_ranked(in) ? n * max(2, in.m - 1) : 0.0f;
+            if (kind == GRP_TREE) return tree_ranked(in) ? n * (in.m == 2 ? 3.0f : (float)max(2, in.m - 1)) : 0.0f;
             return n;
         };
         auto cap = [&](int p) { return group_cap(kind, a.in[p], a.G); };
