@@ -34,7 +34,7 @@ UNIT = "pairs/s"
 N2, M, H, D_VARS = 400_000, 3, 631, 12
 SAMPLE_N2, SAMPLE_H = 40_000, 199        # oracle sample: first 40,000 points, 20,100 directions (about 10 s)
 FLUSH_BYTES = 512 << 20                   # > 129 MB L2
-KERNELS_PER_STEP = 12                     # launches of one single-population selection
+KERNELS_PER_STEP = 10                     # launches of one single-population selection (M <= 5)
 
 
 def parse():
@@ -127,51 +127,7 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# DRAM traffic of k_dom_pref<3> per byte of stored tiles, from one ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum of one launch at
-# 2N=100,000, M=3: 19.00 MB read + 574.31 MB written for 635.79 MB of tiles).
-# The kernel's reads (prefix sets, bucket index, keys) and writes (tiles) grow
-# with the tiles it writes, so the bench scales it by the timed workload's
-# tile bytes. It is reported only while the kernel sources are the ones it
-# was measured on.
-DOM_TRAFFIC_PER_TILE_BYTE = (18_997_504 + 574_313_984) / 635_785_216
-DOM_TRAFFIC_SOURCES_SHA1 = "2fef57b62605552946187e6fbebff2dd5eb9c084"
-DOM_SOURCES = ("k_dominance.cu", "emo_kernels.cuh", "emo_internal.cuh")
-
-
 FP64_NOMINAL_TFLOPS = 1.25
-
-
-def dom_sources_sha1() -> str:
-    import hashlib
-    h = hashlib.sha1()
-    for f in DOM_SOURCES:
-        with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2503_20286_gb300", "csrc", f),
-                  "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()
-
-
-def peel_read_bytes(emo, torch, Ft, F, n_keep: int) -> int:
-    """Bytes the peel must read: every row of the fronts peeled before the last
-    one (rank < l) is read once, 128 bytes per column block at or right of
-    the row's block in lexicographic order (ranks from emo_nd_rank)."""
-    rank, last = emo.emo_nd_rank(Ft, n_keep)
-    torch.cuda.synchronize()
-    r = rank.cpu().numpy()
-    l = int(last.cpu().numpy().reshape(-1)[0])
-    order = np.lexsort(tuple(F[:, k] for k in range(F.shape[1] - 1, -1, -1)))
-    pos = np.empty(F.shape[0], dtype=np.int64)
-    pos[order] = np.arange(F.shape[0])
-    ncb = -(-F.shape[0] // 1024)
-    return int(128 * np.sum(ncb - pos[r < l] // 1024))
-
-
-def triangle_tile_bytes(n2: int) -> int:
-    """Bytes of the stored triangle of D: 4 KB tiles (rb, cb) with cb >= rb / 32."""
-    nrb, ncb = -(-n2 // 32), -(-n2 // 1024)
-    s, t = divmod(nrb, 32)
-    return (nrb * ncb - 32 * (s * (s - 1) // 2) - t * s) * 4096
 
 
 def oneshot_timing(emo, torch, Ft, Rt, n_keep, seed, ws, flush, stream, steps):
@@ -897,17 +853,14 @@ def main():
     ms_per_step = total_ms / args.steps
     value = world * pairs * args.steps / (total_ms / 1e3)
     pk = peaks()
-    dom_ms = statistics.mean(stage_ms.get("dominance", [float("nan")]))
-    # dominance roofline: the kernel must write the triangle of D as 4 KB
-    # tiles; achieved = tile bytes / kernel time against measured HBM copy BW
-    tile_bytes = triangle_tile_bytes(n2)
-    achieved = tile_bytes / (dom_ms / 1e3) / 1e9
-    # peel roofline: the rows of the fronts before the last, read once from HBM
-    peel_ms = statistics.mean(stage_ms.get("peel", [float("nan")]))
-    peel_bytes = peel_read_bytes(emo, torch, Ft, F, n_keep)
-    peel_roofline = {"bound": "hbm", "kernel": "k_peel", "achieved": peel_bytes / (peel_ms / 1e3) / 1e9,
-                     "peak": pk["hbm_gbs"], "unit": "GB/s",
-                     "frac": peel_bytes / (peel_ms / 1e3) / 1e9 / pk["hbm_gbs"], "algorithmic_bytes": peel_bytes}
+    # ranking: the order of the points, then the peeling by the z-order tree (no
+    # dominance matrix up to five objectives). It must read the points and write
+    # their ranks; what it takes beyond that is the chain from front to front.
+    mean_ms = {k: statistics.mean(v) for k, v in stage_ms.items()}
+    rank_ms = sum(mean_ms.get(k, 0.0) for k in ("sort", "colprep", "dominance", "peel"))
+    peel_ms = mean_ms.get("peel", float("nan"))
+    rank_bytes = n2 * (M + 1) * 4
+    achieved = rank_bytes / (peel_ms / 1e3) / 1e9
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
@@ -917,16 +870,13 @@ def main():
                    "l2": f"flushed ({FLUSH_BYTES >> 20} MB write) before every timed step",
                    "parallelism": f"replicas x{world} (independent populations)"},
         "selections_per_s": world * 1e3 / ms_per_step,
-        "dominance_pairs_per_s_kernel": pairs / (dom_ms / 1e3),
-        "stage_ms": {k: statistics.mean(v) for k, v in stage_ms.items()},
-        "roofline": {"bound": "hbm", "kernel": f"k_dom_pref<{M}>", "achieved": achieved,
-                     "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"],
-                     "traffic": (DOM_TRAFFIC_PER_TILE_BYTE * tile_bytes
-                                 if M == 3 and dom_sources_sha1() == DOM_TRAFFIC_SOURCES_SHA1 else None),
-                     "traffic_source": "ncu dram bytes at 2N=100k scaled by tile bytes",
-                     "algorithmic_bytes": tile_bytes,
+        "dominance_pairs_per_s_kernel": pairs / (rank_ms / 1e3),
+        "stage_ms": mean_ms,
+        "roofline": {"bound": "latency", "kernel": f"k_fronts ({M} objectives)", "achieved": achieved,
+                     "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "traffic": None,
+                     "algorithmic_bytes": rank_bytes, "fronts": int(info_h[6]),
+                     "us_per_front": peel_ms * 1e3 / max(1, int(info_h[6])),
                      "peak_source": f"{pk['source']} HBM copy bandwidth"},
-        "peel_roofline": peel_roofline,
         "e2e": {"value": world * pairs / (e2e_ms / 1e3), "unit": UNIT, "ms_per_step": e2e_ms,
                 "h2d_bytes_per_step": int(F.nbytes + R.nbytes), "d2h_bytes_per_step": int(n_keep * 4)},
         "gpu_launches": KERNELS_PER_STEP * args.steps,
