@@ -135,7 +135,7 @@ emo_status emo_dominance(const float* F, int64_t n2, int32_t m, uint32_t* D, int
  * (identical points are the runs of a lexicographic sort). For m <= 5; for
  * larger m it runs the direct kernel of emo_dominance (ws unused). ws:
  * emo_workspace_size(EMO_OP_DOMINANCE_WS, n2, m, 0) bytes, 256-byte aligned
- * (about 0.2 x n2 x m KB: the prefix sets). Non-finite objectives give
+ * (about 0.03 x n2 x m KB: the prefix sets). Non-finite objectives give
  * EMO_ERR_NONFINITE in the workspace status word (the matrix is then
  * undefined).
  */

@@ -1,8 +1,8 @@
 // Set-up, input validation and the lexicographic ordering of the points.
 //
 // The points are put in lexicographic order of (f_1, ..., f_m) by a stable
-// LSD radix sort (8-bit digits of an order-preserving uint32 key, objective
-// m first, objective 1 last). In that order a point can only be dominated by
+// LSD radix sort (8-bit digits of the varying bits of order-preserving uint32
+// keys, objective m first, objective 1 last). In that order a point can only be dominated by
 // points before it (Section IV-A: p dominates q implies f(p) <= f(q)
 // componentwise, hence f(p) <=_lex f(q)), which is what lets the dominance
 // kernel compute and store only the upper triangle of D. Runs of identical
