@@ -96,7 +96,15 @@ __forceinline__ __host__ __device__ bool lex_ordered(const ProbIn& in)
     return !in.ranked && (in.mode == MODE_DOM || in.mode == MODE_HYPE || !tree_ranked(in));
 }
 
-// Per-problem scalars; zeroed by the prep kernel.
+// Members found per front, in three slots taken in turn. The CTAs of a group
+// add to front k's slot between two barriers and read it after the second; the
+// CTA of rank 0 clears the next front's slot while front k is sought. A CTA that
+// leaves a barrier early therefore never adds to, or clears, a slot that one
+// still behind it has to read. (A single running total would: a late reader
+// sees part of the next front in it and leaves the loop alone.)
+__host__ __device__ constexpr int front_slot(int64_t k) { return (int)(k % 3); }
+
+// Per-problem scalars; zeroed by the set-up kernel.
 struct Scal {
     int32_t status;
     int32_t l;
@@ -106,7 +114,7 @@ struct Scal {
     int32_t fallback;
     int32_t nflag;           // points associated by an FP64 scan of more than two references
     int32_t levels;
-    int32_t front_total[2];  // members of the current / next front
+    int32_t front_new[3];    // members of front k in slot k % 3 (see front_slot)
     int32_t idx_buf;         // idx half holding the sorted order
     int32_t lbuf;            // llist half holding the sorted candidate lists
     int32_t nbad;            // points listed for the scan of every reference

@@ -147,23 +147,24 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
     for (int a = gw; a < nnode; a += nw) node_box(a, zstate, zstate);
     if (!group_sync(g, sc, budget)) return false;
 
-    int64_t prev = -1, total = 0;
-    int k_front = 0;
+    int64_t total = 0;  // points ranked
+    int k_front = 0, found = 0;  // members of the front before
     for (;; ++k_front) {
         float* const cur = zstate + (k_front & 1) * state_n;
         float* const nxt = zstate + (~k_front & 1) * state_n;
         // ---- this front's state
         for (int i = tid * 4; i < copied; i += kTreeThreads * 4) front_copy16(s_dyn + i, cur + i);
-        total = ld_volatile(&sc->ranked);
+        if (k_front > 0) found = ld_volatile(&sc->front_new[front_slot(k_front - 1)]);
+        total += found;
+        if (g.rank == 0 && tid == 0) sc->front_new[front_slot(k_front + 1)] = 0;
         if (tid == 0) sm.count = sm.qn = sm.qnext = 0;
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         if (total >= target) break;
-        if (total == prev || k_front >= n2) {  // an empty front before the target: inconsistent
+        if ((k_front > 0 && found == 0) || k_front >= n2) {  // an empty front before the target: inconsistent
             if (tid == 0) set_status(sc, EMO_ERR_INVALID_ARG);
             return false;
         }
-        prev = total;
         // the leaves' state (in global memory: read past L1)
         const float* const llo = (SHARED ? s_dyn : cur) + M * ns;
         const uint32_t* const lmask = reinterpret_cast<const uint32_t*>(llo + M * ls);
@@ -310,7 +311,7 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
 
         // ---- (C) the state of the next front: leaves that lost points, and
         // those whose other parity is a front behind
-        if (tid == 0 && sm.count) atomicAdd(&sc->ranked, sm.count);
+        if (tid == 0 && sm.count) atomicAdd(&sc->front_new[front_slot(k_front)], sm.count);
         for (int i = warp; i < nloc; i += NW) {
             const unsigned gone = *(volatile uint32_t*)&fresh[i], behind = *(volatile uint32_t*)&late[i];
             if (!(gone | behind)) continue;
@@ -339,8 +340,8 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
     if (g.rank == 0 && tid == 0) {
         const int l = k_front - 1;
         sc->l = l;
-        sc->nP = (int32_t)prev;
-        sc->nL = (int32_t)(total - prev);
+        sc->nP = (int32_t)(total - found);
+        sc->nL = found;
         sc->nfronts = l + 1;
         if (d.in.last_rank_out) *d.in.last_rank_out = l;
     }
