@@ -109,7 +109,6 @@ struct Scal {
     int32_t status;
     int32_t l;
     int32_t nP, nL, nS;
-    int32_t ranked;          // points ranked so far
     int32_t nfronts;
     int32_t fallback;
     int32_t nflag;           // points associated by an FP64 scan of more than two references

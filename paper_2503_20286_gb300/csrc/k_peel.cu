@@ -156,18 +156,19 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
         __syncthreads();
         if (tid == 0) {
             d.front_n[cb] = s_newn;
-            atomicAdd(&d.sc->ranked, s_newn);
+            atomicAdd(&d.sc->front_new[front_slot(0)], s_newn);
         }
     }
     if (!group_sync(g, d.sc, budget)) return;
 
-    int64_t prev_total = 0, total = ld_volatile(&d.sc->ranked);
+    int found = ld_volatile(&d.sc->front_new[front_slot(0)]);  // members of front k
+    int64_t total = found;
     int k = 0;
     __shared__ int s_item;
     // (a counter round trip per block pays only across many CTAs)
     const bool dynamic = g.size >= 64 && ncb > 2 * g.size;
     while (total < target) {
-        if (total == prev_total || k >= n2) {  // empty front before the target: inconsistent counts
+        if (found == 0 || k >= n2) {  // empty front before the target: inconsistent counts
             if (tid == 0) set_status(d.sc, EMO_ERR_INVALID_ARG);
             return;
         }
@@ -177,8 +178,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
         int32_t* fw = d.front + (int64_t)nxt * n2p;
         int32_t* fwn = d.front_n + (int64_t)nxt * ncb;
         // the next front's block counter (every CTA left this one's loop
-        // before the last barrier)
-        if (g.rank == 0 && tid == 0) d.wcnt[nxt] = 0;
+        // before the last barrier) and member count
+        if (g.rank == 0 && tid == 0) {
+            d.wcnt[nxt] = 0;
+            d.sc->front_new[front_slot(k + 2)] = 0;
+        }
 
         // prefix of the member counts of every column block
         {
@@ -312,13 +316,13 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
                 __syncthreads();
                 if (tid == 0) {
                     fwn[cb] = s_newn;
-                    atomicAdd(&d.sc->ranked, s_newn - s_base);
+                    atomicAdd(&d.sc->front_new[front_slot(k + 1)], s_newn - s_base);
                 }
             }
         }
         if (!group_sync(g, d.sc, budget)) return;
-        prev_total = total;
-        total = ld_volatile(&d.sc->ranked);
+        found = ld_volatile(&d.sc->front_new[front_slot(k + 1)]);
+        total += found;
         ++k;
     }
 
@@ -326,8 +330,8 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_peel(Plan* plan)
     const int l = k;
     if (g.rank == 0 && tid == 0) {
         d.sc->l = l;
-        d.sc->nP = (int32_t)prev_total;
-        d.sc->nL = (int32_t)(total - prev_total);
+        d.sc->nP = (int32_t)(total - found);
+        d.sc->nL = found;
         d.sc->nfronts = l + 1;
         if (in.last_rank_out) *in.last_rank_out = l;
     }

@@ -113,3 +113,12 @@ def test_front_counts_of_the_tree():
     ops = _accesses(_block(_source("k_fronts.cu"), "for (;; ++k_front)"), "(?:ranked|front_new)", "group_sync")
     assert [k for k, _ in ops].count("read") == 1 and [k for k, _ in ops].count("add") == 1
     assert _reads([], ops) == (0,) + tuple(_added(k) for k in range(4))  # the front before
+
+
+def test_front_counts_of_the_matrix():
+    text = _block(_source("k_peel.cu"), "k_peel(Plan* plan)")
+    loop = _block(text, "while (total < target)")
+    first, ops = (_accesses(t, "(?:ranked|front_new)", "group_sync") for t in (text[:text.index(loop)], loop))
+    assert [k for k, _ in first] == ["add", "barrier", "read"]
+    assert [k for k, _ in ops].count("read") == 1 and [k for k, _ in ops].count("add") == 1
+    assert _reads(first, ops) == (_added(0),) + tuple(_added(k) for k in range(5))
