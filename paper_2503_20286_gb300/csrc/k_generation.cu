@@ -567,6 +567,7 @@ __global__ void __launch_bounds__(kGenThreads) k_igd_near(const float* __restric
         __syncthreads();
         const bool last = i0 + (int64_t)gridDim.y * kTile >= n;
         const int nn = s_near_n;
+        __syncthreads();  // every warp has read the count before the next tile adds to it
         if (nn <= (last ? 0 : kIgdNear - kTile)) continue;  // room for the next tile
         for (int j0 = 0; j0 < nn; j0 += kGenThreads) {
             const int j = j0 + tid;

@@ -122,3 +122,11 @@ def test_front_counts_of_the_matrix():
     assert [k for k, _ in first] == ["add", "barrier", "read"]
     assert [k for k, _ in ops].count("read") == 1 and [k for k, _ in ops].count("add") == 1
     assert _reads(first, ops) == (_added(0),) + tuple(_added(k) for k in range(5))
+
+
+def test_near_points_of_a_tile():
+    """The way from tile to tile of k_igd_near that adds to the list only."""
+    loop = _block(_block(_source("k_generation.cu"), "k_igd_near(const float*"), "for (int64_t i0 =")
+    ops = _accesses(loop[:loop.index("continue;")], "s_near_n", "__syncthreads")
+    assert [k for k, _ in ops][:3] == ["add", "barrier", "read"]
+    assert _reads([], ops) == tuple(sum(_added(q) for q in range(k + 1)) for k in range(5))
