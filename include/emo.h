@@ -436,8 +436,8 @@ emo_status emo_nsga3_generation(float* X, float* F, int64_t n, int64_t d, int32_
  * emo_nsga3_select without a caller workspace, for callers that cannot
  * allocate device memory (a plug-in whose host owns every allocation, a loop
  * that must not enter an allocator, a fixed memory budget). The paper has no
- * counterpart; this is a deployment convenience. The selection runs in an
- * 9 MiB scratch array built into the library (held on every GPU that loads
+ * counterpart; this is a deployment convenience. The selection runs in a
+ * 12 MiB scratch array built into the library (held on every GPU that loads
  * it until the process exits); populations with n2 <= 7168 and n_r <= 7168
  * (any m <= 16) always fit on devices with up to 304 SMs, and n2 <= 8192
  * with n_r <= 8192 (m <= 8) on devices with up to 152 SMs (the workspace

@@ -335,6 +335,13 @@ __host__ __device__ __forceinline__ int fronts_smem_bytes(int64_t n2, int m)
                  (nleaf < front_local(m) ? nleaf : front_local(m)) * (4 + 32 * (m + 1)) * 4);
 }
 
+// Built-in scratch of the allocation-free selection (emo_noalloc.cu). A
+// selection that fitted into 9 MiB while the references were ordered by angle
+// and the prefix sets stored by halves needs up to 11.74 MiB now (the cells of
+// the references' tree, 2 MB from 65,536 references on, and the sets of seven
+// and eight keys).
+constexpr size_t kNoallocBytes = size_t(12) << 20;
+
 // CTA groups of the cooperative kernels: wide (peeling from the matrix,
 // TensorHypE), tree (peeling by the z-order tree), narrow (the others).
 enum GroupKind : int { GRP_NARROW = 0, GRP_WIDE = 1, GRP_TREE = 2 };

@@ -5,7 +5,7 @@
 // a real-time loop that must not enter the driver's allocator, or a process
 // whose memory budget is fixed up front. emo_nsga3_select_noalloc serves them
 // by running the selection in a scratch area that is part of the library
-// image itself: a file-scope device array of kScratchBytes (9 MiB). Every
+// image itself: a file-scope device array of kNoallocBytes (12 MiB). Every
 // GPU on which the library is loaded holds that array until the process
 // exits. Only inputs and outputs come from the caller.
 //
@@ -23,10 +23,10 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = size_t(9) << 20;
+using emo::kNoallocBytes;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[kNoallocBytes];
 
 std::mutex g_scratch_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
@@ -55,10 +55,10 @@ extern "C" emo_status emo_nsga3_select_noalloc(const float* F, int64_t n2, int32
 {
     const size_t need = emo_workspace_size(EMO_OP_NSGA3_SELECT, n2, m, n_r);
     if (need == 0) return EMO_ERR_INVALID_ARG;
-    if (need > kScratchBytes) return EMO_ERR_WORKSPACE;  // population too large for the built-in scratch
+    if (need > kNoallocBytes) return EMO_ERR_WORKSPACE;  // population too large for the built-in scratch
     void* ws = nullptr;
     const emo_status st = scratch_address(&ws);
     if (st != EMO_OK) return st;
-    return emo_nsga3_select(F, n2, m, R, n_r, n_keep, seed, generation, survivors, info, ws, kScratchBytes,
+    return emo_nsga3_select(F, n2, m, R, n_r, n_keep, seed, generation, survivors, info, ws, kNoallocBytes,
                             stream);
 }
