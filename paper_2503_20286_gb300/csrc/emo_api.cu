@@ -966,14 +966,15 @@ emo_status emo_autotune(int32_t m, int64_t n2, const char* cache_path)
         st = EMO_ERR_CUDA;
     } else {
         const int prev_timing = g_timing.exchange(1);
-        // Sum over three selections of the named stages' device times with
-        // shape `sh` forced (the first selection also warms up), or +inf.
+        // Sums of the named stages' device times over three selections with shape
+        // `sh` forced (one more before them warms up): the fastest and the slowest.
+        struct Span { float lo, hi; };
         auto timed = [&](const Shape& sh, std::initializer_list<const char*> stages) {
             {
                 std::lock_guard<std::mutex> lk(g_tune_mu);
                 g_force = sh;
             }
-            float best_ms = INFINITY;
+            Span t{INFINITY, 0.0f};
             for (int rep = 0; rep < 4 && st == EMO_OK; ++rep) {
                 st = emo_nsga3_select((const float*)dF, n2, m, (const float*)dR, (int32_t)n_r, n2 / 2, 1, rep,
                                       (int32_t*)dS, nullptr, dW, wsb, nullptr);
@@ -988,53 +989,41 @@ emo_status emo_autotune(int32_t m, int64_t n2, const char* cache_path)
                 for (int i = 0; i < ns; ++i)
                     for (const char* nm : stages)
                         if (std::strcmp(names[i], nm) == 0) sum += ms[i];
-                if (rep > 0) best_ms = std::min(best_ms, sum);
+                if (rep > 0) t = Span{std::min(t.lo, sum), std::max(t.hi, sum)};
             }
-            return best_ms;
+            return t;
         };
-        // coordinate search, one shape parameter at a time in pipeline order
-        float bms = INFINITY;
-        for (int c = kDomChunkMin; c <= kDomRowChunk && st == EMO_OK; c <<= 1) {
-            Shape t = best;
-            t.dom_chunk = c;
-            const float v = timed(t, {"dominance"});
-            if (v < bms) { bms = v; best.dom_chunk = c; }
-        }
-        bms = INFINITY;
-        for (int w = 0; w <= 1 && st == EMO_OK; ++w) {
-            Shape t = best;
-            t.peel_wave = w;
-            const float v = timed(t, {"peel"});
-            if (v < bms) { bms = v; best.peel_wave = w; }
-        }
-        std::vector<int> caps = {0};
+        // coordinate search, one shape parameter at a time in pipeline order. A
+        // value is taken when its slowest selection beats the fastest one of the
+        // best so far, the default first: what differs by no more than the
+        // repeats do stays as it is.
+        auto search = [&](int Shape::*field, const std::vector<int>& values, std::initializer_list<const char*> stages) {
+            Span least = timed(best, stages);
+            const int start = best.*field;
+            for (int c : values) {
+                if (st != EMO_OK) break;
+                if (c == start) continue;
+                Shape t = best;
+                t.*field = c;
+                const Span v = timed(t, stages);
+                if (st == EMO_OK && v.hi < least.lo) {
+                    least = v;
+                    best.*field = c;
+                }
+            }
+        };
+        std::vector<int> chunks, caps;
+        for (int c = kDomChunkMin; c <= kDomRowChunk; c <<= 1) chunks.push_back(c);
         for (int c = di.G / 2; c >= 1; c /= 2) caps.push_back(c);
-        bms = INFINITY;
-        for (int c : caps) {
-            if (st != EMO_OK) break;
-            Shape t = best;
-            t.cap_wide = c;
-            t.cap_narrow = 0;
-            const float v = timed(t, {"peel"});
-            if (v < bms) { bms = v; best.cap_wide = c; }
+        if (m > kTreeMaxM) {  // (fewer objectives are ranked without the matrix)
+            search(&Shape::dom_chunk, chunks, {"dominance"});
+            search(&Shape::peel_wave, {1 - best.peel_wave}, {"peel"});
         }
-        bms = INFINITY;
-        for (int c : caps) {
-            if (st != EMO_OK) break;
-            if (best.cap_wide > 0 && (c == 0 || c > best.cap_wide)) continue;
-            Shape t = best;
-            t.cap_narrow = c;
-            const float v = timed(t, {"sort", "stats", "csr", "niche", "finish"});
-            if (v < bms) { bms = v; best.cap_narrow = c; }
-        }
-        bms = INFINITY;
-        for (int c : {2, 4, 8, 16, 32}) {
-            if (st != EMO_OK) break;
-            Shape t = best;
-            t.assoc_bps = c;
-            const float v = timed(t, {"assoc"});
-            if (v < bms) { bms = v; best.assoc_bps = c; }
-        }
+        search(&Shape::cap_wide, caps, {"peel"});
+        if (best.cap_wide > 0)  // at most as many
+            caps.erase(std::remove_if(caps.begin(), caps.end(), [&](int c) { return c > best.cap_wide; }), caps.end());
+        search(&Shape::cap_narrow, caps, {"sort", "stats", "csr", "niche", "finish"});
+        search(&Shape::assoc_bps, {2, 4, 8, 16, 32}, {"assoc"});
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
             g_force = Shape{0, 0, -1, -1, -1};
