@@ -367,7 +367,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
     int64_t off = kPlanBytes;
     int max_ncb = 1;
     int fronts_smem = 0;
-    bool any_select = false, any_hype = false, any_tree = false, any_matrix = false, any_lex = false;
+    bool any_select = false, any_hype = false, any_tree = false, any_lex = false;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return EMO_ERR_CUDA;
     for (auto& in : ins) {
@@ -384,8 +384,6 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         if (tree_ranked(in)) {
             any_tree = true;
             fronts_smem = std::max(fronts_smem, fronts_smem_bytes(in.n2, in.m));
-        } else {
-            any_matrix = true;
         }
     }
     if ((int64_t)ws_bytes < off) return EMO_ERR_WORKSPACE;
@@ -447,11 +445,8 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         p = q;
     }
     sm.mark("dominance");
-    if (any_matrix) {
-        int big = 0;
-        for (int p = 1; p < nprob; ++p)
-            if (ins[p].n2 > ins[big].n2) big = p;
-        const bool wave = shape_for(dev, di.sms, ins[big].m, ins[big].n2).peel_wave != 0;
+    if (const int lead = matrix_lead(ins.data(), nprob); lead >= 0) {
+        const bool wave = shape_for(dev, di.sms, ins[lead].m, ins[lead].n2).peel_wave != 0;
         const size_t smem = (size_t)(wave ? peel_wave_smem_bytes(max_ncb) : peel_smem_bytes(max_ncb));
         if (coop(wave ? (const void*)k_peel_wave : (const void*)k_peel, di.G, smem, s, plan) != cudaSuccess)
             return EMO_ERR_CUDA;

@@ -96,6 +96,17 @@ __forceinline__ __host__ __device__ bool lex_ordered(const ProbIn& in)
     return !in.ranked && (in.mode == MODE_DOM || in.mode == MODE_HYPE || !tree_ranked(in));
 }
 
+// The problem whose launch shape the peeling from the matrix takes: the largest
+// of those that are ranked from it (one launch serves them all; the first of
+// equal ones); -1 when there is none.
+inline int matrix_lead(const ProbIn* ins, int n)
+{
+    int lead = -1;
+    for (int p = 0; p < n; ++p)
+        if (!tree_ranked(ins[p]) && (lead < 0 || ins[p].n2 > ins[lead].n2)) lead = p;
+    return lead;
+}
+
 // Members found per front, in three slots taken in turn. The CTAs of a group
 // add to front k's slot between two barriers and read it after the second; the
 // CTA of rank 0 clears the next front's slot while front k is sought. A CTA that
