@@ -472,8 +472,20 @@ __global__ void __launch_bounds__(kAssocWarps * 32, M <= kTreeMaxM ? 3 : 2) k_as
             f[k] = act ? (d.in.F[v * M + k] - sc->z[k]) * sc->inv_a32[k] : 0.0f;
             n2 = fmaf(f[k], f[k], n2);
         }
+        // next to the ideal point: scaled by a power of two (which changes no
+        // angle), so that no square underflows and the error band holds
+        float least = 0.0f;
+        if (n2 < 0x1p-80f) {
+            n2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                f[k] *= 0x1p96f;
+                n2 = fmaf(f[k], f[k], n2);
+            }
+            least = 0x1p-24f;  // (below, the rounding of denormal components counts)
+        }
         const float nrm = sqrtf(n2);
-        const bool bad = act && (!(nrm > 0.0f) || !isfinite(nrm));
+        const bool bad = act && (!(nrm > least) || !isfinite(nrm));
         if (bad && sub == 0) {  // at the ideal point (or overflow): every reference in FP64
             atomicAdd(&sc->nflag, 1);
             d.flagged[atomicAdd(&sc->nbad, 1)] = (int32_t)v;
