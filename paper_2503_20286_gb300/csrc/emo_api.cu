@@ -427,7 +427,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
         sm.mark("rank_in");
         return run_selection_stages(ins, di, plan, dev, s, sm, true, sp.kind);
     }
-    if (any_lex && launch_colprep(plan, di.sms, s, nprob) != cudaSuccess) return EMO_ERR_CUDA;
+    if (any_lex && launch_colprep(plan, di.sms, s) != cudaSuccess) return EMO_ERR_CUDA;
     sm.mark("colprep");
     // dominance: one launch per objective count present
     long long item = 0;
@@ -438,7 +438,7 @@ emo_status run(std::vector<ProbIn>& ins, void* ws, size_t ws_bytes, cudaStream_t
             if (!tree_ranked(ins[q])) hi += dom_items_of(ins[q].n2, ins[q].dom_chunk);
             ++q;
         }
-        if (hi > item && launch_dominance_tri_range(ins[p].m, plan, di.sms, s, item, hi, &plan->dom_ctr[ins[p].m], p, q) !=
+        if (hi > item && launch_dominance_tri_range(ins[p].m, plan, di.sms, s, item, hi, &plan->dom_ctr[ins[p].m]) !=
             cudaSuccess)
             return EMO_ERR_CUDA;
         item = hi;
@@ -1089,8 +1089,10 @@ int32_t emo_device_report(char* buf, int32_t len)
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     out += "; sms " + std::to_string(sms) + "; cooperative " + std::to_string(coop);
     DevInfo di = dev_info();  // also sets the dynamic shared memory limit of k_peel
-    struct K { const char* name; const void* fn; int dyn; };
-    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_order", (const void*)k_order, 0}, {"k_peel", (const void*)k_peel, kPeelDynSmem},
+    struct K { const char* name; const void* fn; int dyn, threads = kCoopThreads; };
+    const K ks[] = {{"k_sort", (const void*)k_sort, 0}, {"k_order", (const void*)k_order, 0},
+                    {"k_fronts", (const void*)k_fronts, kFrontsDynSmem, kTreeThreads},
+                    {"k_peel", (const void*)k_peel, kPeelDynSmem},
                     {"k_stats", (const void*)k_stats, 0}, {"k_csr", (const void*)k_csr, 0},
                     {"k_niche", (const void*)k_niche, 0}, {"k_niche_oneshot", (const void*)k_niche_oneshot, 0},
                     {"k_peel_wave", (const void*)k_peel_wave, kPeelWaveDynSmem},
@@ -1100,7 +1102,7 @@ int32_t emo_device_report(char* buf, int32_t len)
         cudaFuncAttributes fa{};
         int occ = -1;
         cudaError_t e1 = cudaFuncGetAttributes(&fa, k.fn);
-        cudaError_t e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, kCoopThreads, k.dyn);
+        cudaError_t e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.threads, k.dyn);
         out += std::string("; ") + k.name + " regs " + std::to_string(fa.numRegs) + " smem " +
                std::to_string(fa.sharedSizeBytes) + " occ " + std::to_string(occ);
         if (e1 != cudaSuccess || e2 != cudaSuccess)

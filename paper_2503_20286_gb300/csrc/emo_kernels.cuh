@@ -237,9 +237,8 @@ __global__ void k_finish(Plan* plan);
 // Dominance kernels, one instantiation per objective count (k_dominance.cu).
 // The triangle kernel serves items [lo, hi) of the plan through `counter`.
 cudaError_t launch_dominance_tri_range(int m, Plan* plan, int sms, cudaStream_t s, long long lo, long long hi,
-                                       unsigned long long* counter, int pfirst, int plast);
-cudaError_t launch_assoc(Plan* plan, int nprob, const int* m_of, int sms, cudaStream_t s);
-cudaError_t launch_colprep(Plan* plan, int sms, cudaStream_t s, int nprob);
+                                       unsigned long long* counter);
+cudaError_t launch_colprep(Plan* plan, int sms, cudaStream_t s);
 // MODE_DOM (one problem, m <= 5): caller-order keys, prefix sets of every
 // objective, then the full matrix by prefix sets over `nitems` items.
 cudaError_t launch_dominance_caller(int m, Plan* plan, int sms, cudaStream_t s, long long nitems,

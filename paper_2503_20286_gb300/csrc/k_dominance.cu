@@ -151,7 +151,7 @@ __device__ __forceinline__ void segment_sets(unsigned char* blk, const float* s_
     }
 }
 
-__global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int plast)
+__global__ void __launch_bounds__(256) k_colprep(Plan* plan)
 {
     __shared__ float s_v[kColBlock];
     __shared__ uint16_t s_i[kColBlock];
@@ -165,27 +165,27 @@ __global__ void __launch_bounds__(256) k_colprep(Plan* plan, int pfirst, int pla
     auto keys_of = [&](const ProbDev& d) { return d.in.mode == MODE_DOM ? d.in.m : d.in.m - 1; };
     if (tid == 0) {
         long long acc = 0;
-        for (int p = pfirst; p < plast; ++p) {
-            s_first[p - pfirst] = acc;
+        for (int p = 0; p < plan->nprob; ++p) {
+            s_first[p] = acc;
             const ProbDev& d = plan->p[p];
             if (d.colpre && ld_volatile(&d.sc->status) == 0) acc += (long long)d.ncb * keys_of(d);
         }
-        s_first[plast - pfirst] = acc;
+        s_first[plan->nprob] = acc;
     }
     __syncthreads();
     // the items of every problem in one sequence (a batch's small problems
     // together fill the grid)
-    const long long total = s_first[plast - pfirst];
-    int p = pfirst;
+    const long long total = s_first[plan->nprob];
+    int p = 0;
     for (long long it_all = blockIdx.x; it_all < total; it_all += gridDim.x) {
-        while (s_first[p + 1 - pfirst] <= it_all) ++p;
+        while (s_first[p + 1] <= it_all) ++p;
         const ProbDev& d = plan->p[p];
         const bool caller = d.in.mode == MODE_DOM;
         const int K = keys_of(d);
         const float* const kv = caller ? d.ckeys : d.keys;
         const PrefGeom G(K);
         const int ncp1 = kHalf >> G.log_cps;  // checkpoints after the first
-        const long long it = it_all - s_first[p - pfirst];
+        const long long it = it_all - s_first[p];
         const int cb = (int)(it / K), k = (int)(it % K);
         unsigned char* blk = d.colpre + ((int64_t)cb * K + k) * G.obj_bytes;
         for (int q = tid; q < kColBlock; q += blockDim.x) {
@@ -998,7 +998,7 @@ cudaError_t launch_dominance_caller(int m, Plan* plan, int sms, cudaStream_t s, 
     k_dom_keys<<<sms * 2, 256, 0, s>>>(plan);
     cudaError_t e0 = cudaGetLastError();
     if (e0 != cudaSuccess) return e0;
-    e0 = launch_colprep(plan, sms, s, 1);
+    e0 = launch_colprep(plan, sms, s);
     if (e0 != cudaSuccess) return e0;
     switch (m) {
     case 2: return launch_caller_k<2>(plan, sms, s, nitems, counter);
@@ -1013,17 +1013,15 @@ cudaError_t launch_dominance_caller(int m, Plan* plan, int sms, cudaStream_t s, 
 
 // The plan's problems are ordered by m; items of objective count m form one
 // contiguous range served by the m-instantiation.
-cudaError_t launch_colprep(Plan* plan, int sms, cudaStream_t s, int nprob)
+cudaError_t launch_colprep(Plan* plan, int sms, cudaStream_t s)
 {
-    k_colprep<<<sms * 4, 256, 0, s>>>(plan, 0, nprob);
+    k_colprep<<<sms * 4, 256, 0, s>>>(plan);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dominance_tri_range(int m, Plan* plan, int sms, cudaStream_t s, long long lo, long long hi,
-                                       unsigned long long* counter, int pfirst, int plast)
+                                       unsigned long long* counter)
 {
-    (void)pfirst;
-    (void)plast;
     switch (m) {
     case 6: return launch_tri_m<6>(plan, sms, s, lo, hi, counter);
     case 7: return launch_tri_m<7>(plan, sms, s, lo, hi, counter);

@@ -811,9 +811,4 @@ cudaError_t launch_assoc(Plan* plan, int nprob, const int* m_of, int sms, int bl
     return cudaSuccess;
 }
 
-cudaError_t launch_assoc(Plan* plan, int nprob, const int* m_of, int sms, cudaStream_t s)
-{
-    return launch_assoc(plan, nprob, m_of, sms, 8, s);  // the default shape: 8 blocks per SM
-}
-
 }  // namespace emo
