@@ -546,9 +546,9 @@ def autotune_report(emo, torch, dev, flush, stream, steps):
     return {"default": default, "tuned": tuned, "tuned_sizes": len(tuned_keys), "tune_s": tune_s,
             "speedup": {k: default[k] / tuned[k] for k in ("select_ms", "nd_rank_all_fronts_ms", "batch_64_graph_ms")},
             "survivors_and_ranks_identical": same,
-            "tuner": "emo_autotune: dominance item size (m >= 6), peel CTAs per front, other cooperative CTAs, "
+            "tuner": "emo_autotune: dominance item size and peel CTAs per front (m >= 6), other cooperative CTAs, "
                      "association blocks per SM (coordinate search; a value is taken when its slowest of three "
-                     "selections beats the fastest of the best so far)"}
+                     "selections beats the fastest of the best so far by more than 3%)"}
 
 
 def _gpu_select_debug(emo, torch, dev, F, R, n_keep, seed, gen):

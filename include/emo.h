@@ -468,16 +468,16 @@ emo_status emo_get_last_device_status(emo_stream_t stream, int32_t* status_out);
  * architecture, by a coordinate search timed with the stage events on a
  * synthetic population (a sphere-shaped front and n2/2 directions on the
  * simplex), each candidate by three selections, taken when the slowest of
- * them beats the fastest of the best so far (the default first), in this
- * order:
- *   1. for m >= 6 (fewer objectives are ranked without the dominance matrix):
- *      dominance work-item size (row blocks per item: 64 .. 1024) by the
- *      dominance kernel's time; the schedule of the peeling by its time: one
- *      grid barrier per front, or the wavefront (a block's task for front k
- *      starts as soon as every lower column block has finished front k - 1;
- *      no grid barrier);
- *   2. how many CTAs serve the peeling (every CTA, half, a quarter, ... down
- *      to a single CTA) by its time;
+ * them beats the fastest of the best so far (the default first) by more than
+ * 3%, in this order, 1 and 2 for m >= 6 only (fewer objectives are ranked
+ * without the dominance matrix, by as many CTAs as the points need):
+ *   1. dominance work-item size (row blocks per item: 64 .. 1024) by the
+ *      dominance kernel's time;
+ *   2. the schedule of the peeling by its time: one grid barrier per front,
+ *      or the wavefront (a block's task for front k starts as soon as every
+ *      lower column block has finished front k - 1; no grid barrier); then
+ *      how many CTAs serve it (every CTA, half, a quarter, ... down to a
+ *      single CTA);
  *   3. the CTAs of the other cooperative stages (sort, statistics, CSR,
  *      niching, survivors; at most as many as step 2) by their summed time;
  *   4. the association kernel's blocks per SM (2, 4, 8, 16, 32).

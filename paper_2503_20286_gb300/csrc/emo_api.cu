@@ -990,8 +990,9 @@ emo_status emo_autotune(int32_t m, int64_t n2, const char* cache_path)
         };
         // coordinate search, one shape parameter at a time in pipeline order. A
         // value is taken when its slowest selection beats the fastest one of the
-        // best so far, the default first: what differs by no more than the
-        // repeats do stays as it is.
+        // best so far, the default first, by more than 3%: the stage events
+        // resolve about 2 us, and what differs by no more than the repeats do
+        // stays as it is.
         auto search = [&](int Shape::*field, const std::vector<int>& values, std::initializer_list<const char*> stages) {
             Span least = timed(best, stages);
             const int start = best.*field;
@@ -1001,7 +1002,7 @@ emo_status emo_autotune(int32_t m, int64_t n2, const char* cache_path)
                 Shape t = best;
                 t.*field = c;
                 const Span v = timed(t, stages);
-                if (st == EMO_OK && v.hi < least.lo) {
+                if (st == EMO_OK && v.hi * 1.03f < least.lo) {
                     least = v;
                     best.*field = c;
                 }
@@ -1010,11 +1011,15 @@ emo_status emo_autotune(int32_t m, int64_t n2, const char* cache_path)
         std::vector<int> chunks, caps;
         for (int c = kDomChunkMin; c <= kDomRowChunk; c <<= 1) chunks.push_back(c);
         for (int c = di.G / 2; c >= 1; c /= 2) caps.push_back(c);
-        if (m > kTreeMaxM) {  // (fewer objectives are ranked without the matrix)
+        // (fewer objectives are ranked without the matrix, by a group that is no
+        // larger than its leaves need; a cap on it would bind the other groups
+        // too: 20,000 points, a cap of 38 CTAs that the peeling did not notice,
+        // 391 us for a selection, 386 without)
+        if (m > kTreeMaxM) {
             search(&Shape::dom_chunk, chunks, {"dominance"});
             search(&Shape::peel_wave, {1 - best.peel_wave}, {"peel"});
+            search(&Shape::cap_wide, caps, {"peel"});
         }
-        search(&Shape::cap_wide, caps, {"peel"});
         if (best.cap_wide > 0)  // at most as many
             caps.erase(std::remove_if(caps.begin(), caps.end(), [&](int c) { return c > best.cap_wide; }), caps.end());
         search(&Shape::cap_narrow, caps, {"sort", "stats", "csr", "niche", "finish"});

@@ -1,5 +1,6 @@
 """The tuner leaves the shapes of stages that a problem does not run at their
-defaults: up to five objectives nothing builds a dominance matrix."""
+defaults: up to five objectives nothing builds a dominance matrix, and the group that ranks by the
+tree is sized by its leaves."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -25,7 +26,7 @@ def test_tree_ranked_sizes_keep_the_matrix_shapes(m, n2):
     try:
         emo.emo_autotune(m, n2)
         tuned = emo.emo_launch_shape(m, n2)
-        for key in ("dom_rowblocks_per_item", "peel_wavefront"):
+        for key in ("dom_rowblocks_per_item", "peel_wavefront", "peel_ctas"):
             assert tuned[key] == default[key]
     finally:
         emo.emo_autotune_reset()
