@@ -1,10 +1,15 @@
 // Internal definitions of the sm_103a NSGA-III selection library.
 //
 // Data layout in HBM, per population ("problem"):
-//   * points are first put in lexicographic order of their objective vectors
-//     (stable LSD radix sort).  In that order p < q implies that q cannot
+//   * up to five objectives the points are ranked by a two-level tree of
+//     bounding boxes: leaves of 32 points in the order of a grid's Morton cells
+//     (k_order.cu), nodes of 32 leaves (k_fronts.cu). There is no dominance
+//     matrix;
+//   * with more objectives, and for TensorHypE's sample counts and the
+//     caller-order matrix, they are put in lexicographic order of their objective
+//     vectors (stable LSD radix sort).  In that order p < q implies that q cannot
 //     dominate p, so the dominance matrix is strictly upper triangular;
-//   * the triangle is stored as 4 KB tiles of 32 rows x 1024 columns
+//   * that triangle is stored as 4 KB tiles of 32 rows x 1024 columns
 //     (32 rows x 32 uint32 words).  Row block rb = rows [32 rb, 32 rb + 32),
 //     column block cb = columns [1024 cb, 1024 cb + 1024); tile (rb, cb)
 //     exists for cb >= rb / 32.  Tiles of a row block are contiguous; inside
@@ -45,8 +50,10 @@ constexpr int64_t kMaxN2 = int64_t(1) << 21;
 constexpr int32_t kNotRanked = EMO_NOT_RANKED;
 // Ranking without a dominance matrix (k_fronts.cu) up to this many objectives:
 // with more, bounding boxes rule out too little (100,000 points of eight
-// objectives: 5.9 ms by the tree, 3.3 ms by the matrix; 40,000 of five: 0.20
-// and 0.26 ms).
+// objectives: 5.9 ms by the tree, 3.3 ms by the matrix, which has since come
+// down to 0.7 ms; 40,000 of five: 0.20 and 0.26 ms). Six and seven were not
+// measured by the tree; 100,000 points of six on one front take 0.49 ms by the
+// matrix, of five 0.50 ms by the tree.
 constexpr int kTreeMaxM = 5;
 constexpr int kTreeThreads = 1024;         // threads of its peeling kernel
 constexpr int kFrontLeafSmem = 64 * 1024;   // leaf states up to this size are copied to shared memory once per front
@@ -387,7 +394,9 @@ __host__ __device__ inline int64_t layout_problem(const ProbIn& in, int G, char*
     const int64_t nrb = cdiv(n2, 32), ncb = cdiv(n2, kColBlock), n2p = ncb * kColBlock;
     const bool tree = tree_ranked(in), lex = lex_ordered(in);
     // (the tiles' space stays in the size that callers reserve, about n2^2 / 16
-    // bytes, also where the ranks come from the tree and nothing touches it)
+    // bytes, also where the ranks come from the tree and nothing touches it: a
+    // selection's workspace is stated, and tested, to be more than ten times that
+    // of one from given ranks)
     const int64_t ntiles = tiles_before(nrb, ncb);
     int64_t off = 0;
     auto take = [&](int64_t bytes) { int64_t o = off; off = align_up(off + bytes, 256); return o; };
@@ -665,7 +674,7 @@ __device__ __forceinline__ Group group_of(const Plan* plan, GroupKind kind)
 // barrier is one atomic plus the poll that sees the last arrival (the
 // former generation barrier took an extra read, an exchange, a fence and a
 // back-off: ranking 20,001 points in 46 fronts 513 -> 462 us, a selection of
-// 184 points with every group at 152 CTAs 332 -> 289 us.
+// 184 points with every group at 152 CTAs 332 -> 289 us).
 __device__ inline bool group_sync(const Group& g, Scal* sc, long long budget)
 {
     __shared__ int s_ok;

@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(kGenThreads) k_gather_rows(const float* __rest
 //     far less than what 2 rad lets in.
 // Measured at n = 200,000, n_ref = 200,028, m = 3: 66.5 ms for a thread per
 // reference point over every pair with runtime m (the former kernel),
-// grouped 0.30 in a warm loop: near 0.25 (the groups that straddle two patches of the front are its
-// tail), centre 0.034, ordering 0.05.
+// grouped 0.30 in a warm loop: near 0.22 (the groups that straddle two patches
+// of the front are its tail), centre 0.034, ordering 0.05.
 constexpr int kIgdGroup = 128;     // reference points per group
 constexpr int kIgdGroups = 8;      // groups per block
 constexpr int kIgdSample = 8;      // every kIgdSample-th point bounds d_c
@@ -245,7 +245,11 @@ constexpr int kIgdStage = 128;     // candidates compared at once
 // The grouped route costs about 75 us before the first comparison; the direct
 // one grows with n n_ref. Measured (direct / grouped, us): n = 65,536, n_ref =
 // 8,192 (5.4e8 pairs) 96 / 105 at m = 2, 131 / 117 at m = 3, 235 / 296 at m = 5,
-// 1623 / 1300 at m = 8; n = n_ref = 8,192 (6.7e7 pairs) 33 / 84 at m = 3.
+// 1623 / 1300 at m = 8; n = n_ref = 8,192 (6.7e7 pairs) 33 / 84 at m = 3. One
+// line for every m: that of m = 3, for m = 8 it would lie lower. Where the skipping
+// rules nothing out (every point about equally far from a group's members) the
+// grouped route loses instead: n = n_ref = 200,000, m = 3, 9.9 / 14.3 ms (9.9 /
+// 0.5 near the front), n = n_ref = 50,000 0.56 / 1.00 ms (0.56 / 0.19).
 constexpr int64_t kIgdMinRefs = 1024;
 constexpr double kIgdMinPairs = 7e8;
 

@@ -10,11 +10,11 @@
 //   (C) c_i = points weakly dominating S_i, from the column-block prefix sets
 //       of the dominance stage (see the kernel);
 //   k_hype phase 1 (cooperative):
-//       the weights alpha_c for c <= k (one thread, in order: lambda_1 = 1,
-//       lambda_c = (k - c + 1) / (n2 - c + 1), alpha_c = (lambda_1 ...
-//       lambda_c) / c; alpha_c = 0 beyond k);
-//   (D) each point of L (one warp, samples staged in shared memory): its
-//       contribution, vol / s times the sum of alpha_{c_i} over the samples
+//       the weights alpha_c for c <= k (lambda_1 = 1, lambda_c =
+//       (k - c + 1) / (n2 - c + 1), alpha_c = (lambda_1 ... lambda_c) / c,
+//       alpha_c = 0 beyond k; the chain of products in order by one thread);
+//   (D) the points of L, two to a warp (samples staged in shared memory): each
+//       one's contribution, vol / s times the sum of alpha_{c_i} over the samples
 //       it dominates in sample order (double);
 //   (E) L sorted stably by (contribution descending) with 64-bit radix passes;
 //       its first n_keep - |P| points are flagged as survivors.

@@ -2,8 +2,9 @@
 //
 // The points are put in lexicographic order of (f_1, ..., f_m) by a stable
 // LSD radix sort (8-bit digits of the varying bits of order-preserving uint32
-// keys, objective m first, objective 1 last). In that order a point can only be dominated by
-// points before it (Section IV-A: p dominates q implies f(p) <= f(q)
+// keys, objective m first, objective 1 last) where the dominance matrix or the
+// prefix sets are built (lex_ordered). In that order a point can only be dominated
+// by points before it (Section IV-A: p dominates q implies f(p) <= f(q)
 // componentwise, hence f(p) <=_lex f(q)), which is what lets the dominance
 // kernel compute and store only the upper triangle of D. Runs of identical
 // objective vectors (which never dominate each other) are recorded so the
@@ -13,8 +14,9 @@
 
 namespace emo {
 
-// One thread per problem: carve the workspace, zero the scalars; thread 0
-// then splits the cooperative grid into CTA groups and counts work items.
+// One thread per problem carves its workspace, the warps zero the scalars, a
+// warp per kind splits the cooperative grid into CTA groups, and one more thread
+// counts the work items.
 __global__ void k_setup(SetupArgs a, SplitArgs sp, Plan* plan, char* ws)
 {
     const int t = threadIdx.x;

@@ -9,7 +9,7 @@
 //   * ASF extreme points: an FP32 pass bounds the minimum, points within the
 //     FP32 error band are re-evaluated in FP64;
 //   * hyperplane intercepts: Gaussian elimination with partial pivoting in
-//     FP64 on one thread (m <= 16), nadir fallback;
+//     FP64 on one warp, a lane per row (m <= 16), nadir fallback;
 //   * association: an FP32 search keeps the three smallest distances; references
 //     whose distance lies within a rigorous error band of the best are
 //     re-evaluated with the FP64 perpendicular distance d^2 = sum (f_k - t r_k)^2,
@@ -331,9 +331,9 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_stats(Plan* plan)
 // unit direction, c and R the ball and b the chord of the best angle (plus a
 // margin). A leaf's 32 references pass through shared memory.
 // Bound by issue and the latency of the leaves' tests. Measured (association
-// and decision together): 200,864 points on 200,028 references, m = 3, 0.33 ms
+// and decision together): 200,864 points on 200,028 references, m = 3, 0.27 ms
 // (0.43 ms by a scan outward from each point's polar angle); 22,170 points on
-// 20,475 references, m = 5, 0.26 ms (0.79 ms visiting every reference); 10,056
+// 20,475 references, m = 5, 0.23 ms (0.79 ms visiting every reference); 10,056
 // on 10,011, m = 3, 53 us (92 us).
 //
 // Error band of the FP32 distance (relative to |f|), two evaluations:
