@@ -120,7 +120,7 @@ inline int matrix_lead(const ProbIn* ins, int n)
 // leaves a barrier early therefore never adds to, or clears, a slot that one
 // still behind it has to read. (A single running total would: a late reader
 // sees part of the next front in it and leaves the loop alone.)
-__host__ __device__ constexpr int front_slot(int64_t k) { return (int)(k % 3); }
+__host__ __device__ constexpr int front_slot(int k) { return (int)((unsigned)k % 3u); }
 
 // Per-problem scalars; zeroed by the set-up kernel.
 struct Scal {

@@ -67,7 +67,7 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
     const int64_t n2 = d.in.n2;
     const int nleaf = d.nleaf, nnode = d.nnode, ls = d.nleafp, ns = d.nnodep;
     const int64_t zs = (int64_t)nleaf * 32;
-    const int64_t target = d.in.n_keep > 0 ? d.in.n_keep : n2;
+    const int target = (int)(d.in.n_keep > 0 ? d.in.n_keep : n2);
     Scal* const sc = d.sc;
     const float* const zp = d.zpts;
     int32_t* const rank_s = d.rank_s;
@@ -147,8 +147,7 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
     for (int a = gw; a < nnode; a += nw) node_box(a, zstate, zstate);
     if (!group_sync(g, sc, budget)) return false;
 
-    int64_t total = 0;  // points ranked
-    int k_front = 0, found = 0;  // members of the front before
+    int k_front = 0, found = 0, total = 0;  // members of the front before, points ranked
     for (;; ++k_front) {
         float* const cur = zstate + (k_front & 1) * state_n;
         float* const nxt = zstate + (~k_front & 1) * state_n;
@@ -340,7 +339,7 @@ __device__ __noinline__ bool peel_tree(const ProbDev& d, const Group& g, long lo
     if (g.rank == 0 && tid == 0) {
         const int l = k_front - 1;
         sc->l = l;
-        sc->nP = (int32_t)(total - found);
+        sc->nP = total - found;
         sc->nL = found;
         sc->nfronts = l + 1;
         if (d.in.last_rank_out) *d.in.last_rank_out = l;
