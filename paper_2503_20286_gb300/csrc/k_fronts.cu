@@ -28,8 +28,8 @@
 // Bound: latency -- a front costs one barrier (1.1 us), the state's way through
 // L2 and the longest search of any warp. Measured against the tiles of the
 // dominance matrix (set-up, matrix and peel): 400,000 points of three
-// objectives to their 37th front 0.84 ms (3.36 ms), 20,001 points, all 46
-// fronts 0.31 ms (0.43 ms), 40,000 points of five objectives 0.20 ms (0.26 ms).
+// objectives to their 37th front 0.88 ms (3.36 ms), 20,001 points, all 46
+// fronts 0.30 ms (0.43 ms), 40,000 points of five objectives 0.20 ms (0.26 ms).
 // Also tried: one warp walking for all searching points of a leaf together
 // (their union of boxes makes the slowest warp 2-4 times slower); the boxes of
 // four nodes and the points of four leaves loaded at once (more instructions
